@@ -13,6 +13,7 @@
 
 #include "glbe.h"
 #include "glbe_internal.h"
+#include "glbe_residual.cuh"
 
 using namespace glbe;
 
@@ -273,83 +274,50 @@ StepParams glbe::make_step_params(const glbe_params* p)
 
 namespace {
 
-constexpr int FIN_THREADS = 1024;
+// Reduction of a residual step's partials [k][block] into the record.  Warp k
+// of every block sums row k of the block's chunk; with more than one block the
+// chunk sums go to row 7 of the partials (unused by the step) and the block
+// that arrives last sums those, so one launch does it all.  Arrivals are
+// counted in the last word of the record, which every record leaves at zero
+// (atomicInc wraps it back there itself).  Chunks of 256 partials: eight
+// additions of a warp per row, then as many blocks as the grid needs (512 for
+// the 512 x 256 x 256 duct), and at most 16 more per row in the last block.
+constexpr int FIN_THREADS = 256;
+constexpr unsigned FIN_CHUNK = 256;
 
-__global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(const double* __restrict__ partials, unsigned nblocks,
-                                                               double mass0, long long* t_dev, double* record,
-                                                               double* hist, unsigned long long* hist_count,
-                                                               unsigned hist_cap, int* stop, const double* tol)
+__global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(double* __restrict__ partials, unsigned nblocks,
+                                                               const RecordOut out)
 {
-    if (*stop) return;   // a solve already converged: the chunk's remaining work is skipped
-    __shared__ double sh[7][FIN_THREADS / 32];
+    if (*out.stop) return;   // a solve already converged: the chunk's remaining work is skipped
+    __shared__ double tot[RES_SUMS];
+    __shared__ int last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < 7; ++k) {
-        // partials are [k][block]: consecutive threads read consecutive blocks
-        const double* pk = partials + (size_t)k * nblocks;
-        double s = 0.0;
-        for (unsigned b = threadIdx.x; b < nblocks; b += FIN_THREADS) s += pk[b];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) sh[k][warp] = s;
+    const unsigned G = gridDim.x;
+    double* const stage = partials + (size_t)RES_SUMS * nblocks;
+    if (warp < RES_SUMS) {
+        const unsigned b0 = blockIdx.x * FIN_CHUNK, b1 = b0 + FIN_CHUNK < nblocks ? b0 + FIN_CHUNK : nblocks;
+        const double v = partial_row_sum(partials + (size_t)warp * nblocks, b0, b1);
+        if (lane == 0) {
+            if (G == 1) tot[warp] = v;
+            else stage[(size_t)warp * G + blockIdx.x] = v;
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot[7];
-        for (int k = 0; k < 7; ++k) {
-            double s = 0.0;
-            for (int w = 0; w < FIN_THREADS / 32; ++w) s += sh[k][w];
-            tot[k] = s;
-        }
-        const double num = tot[0], den = tot[1];
-        const double r = den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0);
-        const long long t = *t_dev;
-        double rec[RECORD_STRIDE] = {0};
-        rec[0] = (double)t;
-        rec[1] = r;
-        rec[2] = num;
-        rec[3] = den;
-        rec[4] = mass0 + tot[2];
-        rec[5] = tot[3];
-        rec[6] = tot[4];
-        rec[7] = tot[5];
-        rec[8] = tot[6];
-        for (int k = 0; k < RECORD_STRIDE; ++k) record[k] = rec[k];
-        const unsigned long long c = *hist_count;
-        double* h = hist + (size_t)(c % hist_cap) * RECORD_STRIDE;
-        for (int k = 0; k < RECORD_STRIDE; ++k) h[k] = rec[k];
-        *hist_count = c + 1;
-        *t_dev = t + 10;
-        if ((*tol > 0.0 && r <= *tol) || rec[8] > 0.0 || !isfinite(r)) *stop = 1;
-    }
-}
-
-// First stage of the residual reduction for large grids: block b sums the
-// partials of blocks [b*chunk, (b+1)*chunk) of the step (fixed order) into
-// row 7 of the partials, which the step leaves unused: out[k][b].
-constexpr int RED_THREADS = 256;
-
-__global__ void __launch_bounds__(RED_THREADS) partial_reduce_kernel(const double* __restrict__ partials,
-                                                                     unsigned nblocks, unsigned fb, double* out,
-                                                                     const int* stop)
-{
-    if (*stop) return;
-    __shared__ double sh[RED_THREADS / 32];
-    const unsigned chunk = (nblocks + fb - 1) / fb;
-    const unsigned b0 = blockIdx.x * chunk, b1 = b0 + chunk < nblocks ? b0 + chunk : nblocks;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < 7; ++k) {
-        const double* pk = partials + (size_t)k * nblocks;
-        double s = 0.0;
-        for (unsigned b = b0 + threadIdx.x; b < b1; b += RED_THREADS) s += pk[b];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) sh[warp] = s;
-        __syncthreads();
+    if (G > 1) {
         if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < RED_THREADS / 32; ++w) t += sh[w];
-            out[(size_t)k * fb + blockIdx.x] = t;
+            __threadfence();
+            last = atomicInc(reinterpret_cast<unsigned*>(out.record + RECORD_STRIDE - 1), G - 1) == G - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!last) return;
+        if (warp < RES_SUMS) {
+            const double v = partial_row_sum(stage + (size_t)warp * G, 0, G);
+            if (lane == 0) tot[warp] = v;
         }
         __syncthreads();
     }
+    if (threadIdx.x == 0) write_record(out, tot, *out.t_dev);
 }
 
 __global__ void misc_set_kernel(long long* t_dev, long long t, int* stop, int stop_v, double* tol, double tol_v,
@@ -486,25 +454,12 @@ glbe_status ctx_view(glbe_ctx* c, CtxView* v)
     return GLBE_OK;
 }
 
-cudaError_t launch_finalize(const double* partials, unsigned nblocks, double mass0, long long* t_dev, double* record,
+cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, long long* t_dev, double* record,
                             double* hist, unsigned long long* hist_count, unsigned hist_cap, int* stop,
                             const double* tol, cudaStream_t st)
 {
-    // large grids: a first stage over many blocks (one SM alone reads the
-    // 7 x nblocks partials at a fraction of the HBM bandwidth), its results
-    // in the unused row 7 of the partials; then the one-block finalize
-    constexpr unsigned PER_BLOCK = 512;
-    if (nblocks >= 2 * PER_BLOCK) {
-        unsigned fb = nblocks / PER_BLOCK;
-        if (7 * fb > nblocks) fb = nblocks / 7;
-        double* row7 = const_cast<double*>(partials) + (size_t)7 * nblocks;
-        partial_reduce_kernel<<<fb, RED_THREADS, 0, st>>>(partials, nblocks, fb, row7, stop);
-        finalize_kernel<<<1, FIN_THREADS, 0, st>>>(row7, fb, mass0, t_dev, record, hist, hist_count, hist_cap, stop,
-                                                   tol);
-    } else {
-        finalize_kernel<<<1, FIN_THREADS, 0, st>>>(partials, nblocks, mass0, t_dev, record, hist, hist_count,
-                                                   hist_cap, stop, tol);
-    }
+    const RecordOut out{record, hist, hist_count, hist_cap, t_dev, stop, tol, mass0};
+    finalize_kernel<<<(nblocks + FIN_CHUNK - 1) / FIN_CHUNK, FIN_THREADS, 0, st>>>(partials, nblocks, out);
     return cudaGetLastError();
 }
 }  // namespace glbe

@@ -160,8 +160,10 @@ cudaError_t launch_set_state_t(bool mhd, const StepParams& p, void* fsrc, void* 
 // the record to the history ring hist[(count % cap) * RECORD_STRIDE].
 constexpr int RECORD_STRIDE = 16;
 // The reduction also raises *stop when r <= *tol (tol > 0) or a velocity is
-// non-finite, and does nothing once *stop is set.
-cudaError_t launch_finalize(const double* partials, unsigned nblocks, double mass0, long long* t_dev,
+// non-finite, and does nothing once *stop is set.  Row 7 of the partials is its
+// scratch; the last word of the record counts its blocks and has to be zero
+// on entry (it is again on exit).
+cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, long long* t_dev,
                             double* record, double* hist, unsigned long long* hist_count, unsigned hist_cap,
                             int* stop, const double* tol, cudaStream_t st);
 
