@@ -1413,27 +1413,19 @@ __device__ __forceinline__ void coupled_induction_pass(const StepParams& p, cons
     induction_from_sources<ST>(p, b, n, d, dl, q, ql);
 }
 
-// Pass 1 of the two-pass coupled update from the gathered populations of
-// node n: rho and m, the induction part, and the stores of g~ and of this
-// step's Lorentz force.
+// 1/rho and m of a node's gathered f, as node_update forms them.
 template <int ST>
-__device__ __forceinline__ void induction_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n,
-                                                      const float (&d)[19], const float (&dl)[19],
-                                                      const float (&q)[21], const float (&ql)[21])
+__device__ __forceinline__ void node_momentum(const StepParams& p, const float (&d)[19], const float (&dl)[19],
+                                              float& rho_inv, float& mx, float& my, float& mz)
 {
-    using S = Store<ST>;
-    using T = typename S::T;
     constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
-    const size_t N = p.N;
-    const NodeIn<float> in = node_inputs<true, MODE_STEP>(p, b, n);
-    // rho and m as node_update forms them
     NodeMoments<float, PRECISE> mm;
     if constexpr (PRECISE) {
         float dh[19], dlo[19];
 #pragma unroll
         for (int a = 0; a < 19; ++a) {
             split_exact(d[a], dh[a], dlo[a]);
-            if constexpr (S::COMP) dlo[a] += dl[a];
+            if constexpr (Store<ST>::COMP) dlo[a] += dl[a];
         }
         mm.H = linear_moments(dh);
         mm.L = linear_moments(dlo);
@@ -1441,14 +1433,21 @@ __device__ __forceinline__ void induction_from_sources(const StepParams& p, cons
         mm.H = linear_moments(d);
     }
     const float rho = p.rho0 + mm.drho();
-    const float rho_inv = vrcp(rho);
-    const float mx = PRECISE ? mm.H.mx + mm.L.mx : mm.H.mx;
-    const float my = PRECISE ? mm.H.my + mm.L.my : mm.H.my;
-    const float mz = PRECISE ? mm.H.mz + mm.L.mz : mm.H.mz;
-    float og[21];
-    NodeMacro<float> mac;
-    induction_collide<float, PRECISE, S::COMP>(p, q, ql, og, rho_inv, mx, my, mz, in.Fx, in.Fy, in.Fz, in.FLx,
-                                              in.FLy, in.FLz, mac);
+    rho_inv = vrcp(rho);
+    mx = PRECISE ? mm.H.mx + mm.L.mx : mm.H.mx;
+    my = PRECISE ? mm.H.my + mm.L.my : mm.H.my;
+    mz = PRECISE ? mm.H.mz + mm.L.mz : mm.H.mz;
+}
+
+// g~ = g + og into node n's own slots, and this step's Lorentz force.
+template <int ST>
+__device__ __forceinline__ void store_induction(const StepParams& p, const StepBuffers& b, uint32_t n,
+                                                const float (&q)[21], const float (&ql)[21], const float (&og)[21],
+                                                float FLx, float FLy, float FLz)
+{
+    using S = Store<ST>;
+    using T = typename S::T;
+    const size_t N = p.N;
     T* __restrict__ gd = static_cast<T*>(b.gdst);
     if constexpr (S::COMP) {
         __half* __restrict__ gdl = reinterpret_cast<__half*>(gd + 21 * N);
@@ -1463,9 +1462,28 @@ __device__ __forceinline__ void induction_from_sources(const StepParams& p, cons
 #pragma unroll
         for (int a = 0; a < 21; ++a) gd[(size_t)a * N + n] = S::cv(toscale<ST>(p, q[a] + og[a]));
     }
-    b.FL[n] = mac.FLx;
-    b.FL[N + n] = mac.FLy;
-    b.FL[2 * N + n] = mac.FLz;
+    b.FL[n] = FLx;
+    b.FL[N + n] = FLy;
+    b.FL[2 * N + n] = FLz;
+}
+
+// Pass 1 of the two-pass coupled update from the gathered populations of
+// node n: rho and m, the induction part, and the stores of g~ and of this
+// step's Lorentz force.
+template <int ST>
+__device__ __forceinline__ void induction_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n,
+                                                      const float (&d)[19], const float (&dl)[19],
+                                                      const float (&q)[21], const float (&ql)[21])
+{
+    constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
+    const NodeIn<float> in = node_inputs<true, MODE_STEP>(p, b, n);
+    float rho_inv, mx, my, mz;
+    node_momentum<ST>(p, d, dl, rho_inv, mx, my, mz);
+    float og[21];
+    NodeMacro<float> mac;
+    induction_collide<float, PRECISE, Store<ST>::COMP>(p, q, ql, og, rho_inv, mx, my, mz, in.Fx, in.Fy, in.Fz, in.FLx,
+                                                      in.FLy, in.FLz, mac);
+    store_induction<ST>(p, b, n, q, ql, og, mac.FLx, mac.FLy, mac.FLz);
 }
 
 // The update of fluid node n from its gathered pre-collision populations
