@@ -192,7 +192,11 @@ glbe_status glbe_set_force(glbe_ctx* ctx, const float* d_F);
 glbe_status glbe_set_force_host(glbe_ctx* ctx, const float* h_F);
 
 /* Advances n >= 0 time steps (one fused kernel per step; the residual is
- * evaluated inside the step that collides a level t with t % 10 == 0). */
+ * evaluated inside the step that collides a level t with t % 10 == 0).  With
+ * the automatic kernel form, small grids (up to about 350,000 nodes) take
+ * n >= 2 steps in one launch whose blocks stay resident and meet at a bounded
+ * barrier between levels: the same states bit for bit.  Should a wait run out,
+ * the next call that synchronises returns GLBE_ERR_TIMEOUT. */
 glbe_status glbe_step_n(glbe_ctx* ctx, long n);
 
 /* Synchronises the stream and returns the latest residual evaluation.
@@ -205,7 +209,8 @@ glbe_status glbe_residual(glbe_ctx* ctx, glbe_residual_info* out);
 glbe_status glbe_history(glbe_ctx* ctx, glbe_residual_info* out, long cap, long* n);
 
 /* Time-marches until r(t) <= tol (t a multiple of 10) or max_steps steps have
- * been taken, replaying a CUDA graph of 10-step chunks.  *steps_out = time
+ * been taken, replaying a CUDA graph of 10-step chunks (small grids: resident
+ * launches, see glbe_step_n).  *steps_out = time
  * level t of the converged residual (or the level reached), *r_out = r(t).
  * GLBE_ERR_TIMEOUT if max_steps was reached first, GLBE_ERR_DIVERGED on
  * NaN/Inf.  Synchronises the stream. */

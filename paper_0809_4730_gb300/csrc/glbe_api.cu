@@ -354,6 +354,9 @@ struct glbe_ctx {
     long long* t_dev;
     int* stop_dev;
     double* tol_dev;
+    unsigned* res_bar;       // barrier words of the resident march (count, generation, error)
+    ResidentPlan res;        // form 0: steps are launched one by one
+    bool res_used;           // a resident march was launched since the error flag was last read
     unsigned* sr_ctr;   // [2] seeds of stochastic rounding, read by the step of parity t & 1
     double mass0;   // rho0 x number of fluid nodes
     long t;         // current time level
@@ -402,6 +405,87 @@ StepBuffers buffers_for(glbe_ctx* c, long t)
     b.sr_par = s;
     b.sr_seed = 0;
     return b;
+}
+
+// The resident march serves the automatic kernel form of the MRT collision in
+// the plainly rounded storage types, without box or lid.
+ResidentPlan plan_resident(const glbe_ctx* c)
+{
+    ResidentPlan r{0, 0, 0, 0, 0};
+    if (c->prm.variant != 0 || c->prm.collision != 0 || c->sp.cavity) return r;
+    const bool mhd = c->prm.induction;
+    cudaError_t e;
+    switch (c->prm.storage) {
+    case GLBE_F32: e = resident_plan<ST_F32>(mhd, c->sp, &r); break;
+    case GLBE_F32C: e = resident_plan<ST_F32C>(mhd, c->sp, &r); break;
+    case GLBE_BF16: e = resident_plan<ST_BF16>(mhd, c->sp, &r); break;
+    case GLBE_F16: e = resident_plan<ST_F16>(mhd, c->sp, &r); break;
+    default: return r;
+    }
+    if (e != cudaSuccess) {   // no plan: single launches, which report what is wrong
+        cudaGetLastError();
+        r.form = 0;
+    }
+    return r;
+}
+
+// Enqueues n >= 1 steps from level c->t as one resident march on the
+// context's stream (solve: with the stop test of tolerance tol).  The host's
+// levels are those of a march that takes every step.
+glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
+{
+    ResidentMarch m{};
+    for (int k = 0; k < 2; ++k) {
+        m.f[k] = c->f[k];
+        m.g[k] = c->g[k];
+    }
+    m.FL = c->FL;
+    m.Ffield = c->Ffield;
+    m.usnap = c->usnap;
+    m.partials = c->partials;
+    m.snap_lo = snap_rows(c->prm.storage) == 6 ? 1 : 0;
+    const long first = (c->t + 9) / 10 * 10;        // first residual level of the march
+    m.have_snap = c->t_snap >= 0 && c->t_snap == first - 10;
+    m.t0 = c->t;
+    m.nsteps = n;
+    m.solve = solve ? 1 : 0;
+    m.tol = tol;
+    m.out = RecordOut{c->record, c->hist, c->hist_count, HIST_CAP, c->t_dev, c->stop_dev, c->tol_dev, c->mass0};
+    m.bar = c->res_bar;
+    const bool mhd = c->prm.induction;
+    cudaError_t e;
+    switch (c->prm.storage) {
+    case GLBE_F32: e = resident_march<ST_F32>(mhd, c->sp, m, c->res, c->stream); break;
+    case GLBE_BF16: e = resident_march<ST_BF16>(mhd, c->sp, m, c->res, c->stream); break;
+    case GLBE_F16: e = resident_march<ST_F16>(mhd, c->sp, m, c->res, c->stream); break;
+    default: e = resident_march<ST_F32C>(mhd, c->sp, m, c->res, c->stream); break;
+    }
+    GLBE_CUDA(e, "resident march");
+    c->res_used = true;
+    if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
+    c->t += n;
+    return GLBE_OK;
+}
+
+// Waits for the stream and reports whether a barrier wait of a resident march
+// ran out; stop (may be NULL) receives the march's stop flag.  One copy of the
+// control words, on the context's own stream.
+glbe_status sync_control(glbe_ctx* c, int* stop)
+{
+    const bool resident = c->res_used && c->res.form >= 2;
+    c->res_used = false;
+    char misc[64] = {0};
+    if (stop || resident)
+        GLBE_CUDA(cudaMemcpyAsync(misc, c->ws + c->L.misc, sizeof misc, cudaMemcpyDeviceToHost, c->stream),
+                  "control words");
+    GLBE_CUDA(cudaStreamSynchronize(c->stream), "sync");
+    if (stop) std::memcpy(stop, misc + ((const char*)c->stop_dev - (c->ws + c->L.misc)), sizeof *stop);
+    if (!resident) return GLBE_OK;
+    unsigned err = 0;
+    std::memcpy(&err, misc + ((const char*)(c->res_bar + 2) - (c->ws + c->L.misc)), sizeof err);
+    if (!err) return GLBE_OK;
+    GLBE_CUDA(cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream), "resident march reset");
+    return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
 }
 
 // Enqueues the step from level c->t to c->t + 1 on stream st.
@@ -543,6 +627,9 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     c->tol_dev = reinterpret_cast<double*>(misc + 16);
     c->stop_dev = reinterpret_cast<int*>(misc + 24);
     c->sr_ctr = reinterpret_cast<unsigned*>(misc + 32);
+    c->res_bar = reinterpret_cast<unsigned*>(misc + 40);
+    c->res = plan_resident(c);
+    c->res_used = false;
     c->mass0 = p->rho0 * (double)fluid_nodes(p);   // planes on walls and ghost planes excluded
     c->t = 0;
     c->t_snap = -1;
@@ -556,7 +643,8 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     cudaError_t e = cudaMemsetAsync(c->ws, 0, L.usnap, c->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->ws + L.usnap, 0, snap_rows(p->storage) * c->N * sizeof(float), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->sr_ctr, 0, 2 * sizeof(unsigned), c->stream);
+    // the seeds and the barrier words behind them
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->sr_ctr, 0, 5 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess && c->sp.cavity) {   // the lid's links of the first gather (see lid_init_kernel)
         if (p->storage == GLBE_F32) e = launch_lid_init_t<ST_F32>(c->sp, c->f[0], c->stream);
         else if (p->storage == GLBE_F32C) e = launch_lid_init_t<ST_F32C>(c->sp, c->f[0], c->stream);
@@ -642,6 +730,7 @@ glbe_status glbe_step_n(glbe_ctx* c, long n)
     NvtxRange range_("glbe_step_n");
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(GLBE_ERR_ARG, "n must be >= 0");
+    if (c->res.form && n >= 2) return enqueue_resident(c, n, false, 0.0);
     for (long k = 0; k < n; ++k) {
         glbe_status s = enqueue_step(c, c->stream, nullptr);
         if (s != GLBE_OK) return s;
@@ -661,13 +750,14 @@ glbe_status glbe_sync(glbe_ctx* c)
     default: break;
     }
     if (waited_out) return fail(GLBE_ERR_TIMEOUT, "a pipeline wait of the TMA-staged step kernel ran out");
-    return GLBE_OK;
+    return sync_control(c, nullptr);
 }
 
 static glbe_status read_record(glbe_ctx* c, glbe_residual_info* out)
 {
     double rec[RECORD_STRIDE];
-    GLBE_CUDA(cudaStreamSynchronize(c->stream), "residual sync");
+    const glbe_status rs = sync_control(c, nullptr);
+    if (rs != GLBE_OK) return rs;
     GLBE_CUDA(cudaMemcpy(rec, c->record, sizeof rec, cudaMemcpyDeviceToHost), "residual read");
     out->t = (long)rec[0];
     out->r = rec[1];
@@ -759,22 +849,36 @@ glbe_status glbe_solve(glbe_ctx* c, double tol, long max_steps, long* steps_out,
     if (max_steps < 0) return fail(GLBE_ERR_ARG, "max_steps must be >= 0");
     const long t_end = c->t + max_steps;
     // align: level a multiple of 10 with a snapshot of the previous multiple of 10
-    while (!(c->t % 10 == 0 && c->t_snap >= 0 && c->t_snap == c->t - 10) && c->t < t_end) {
-        glbe_status s = enqueue_step(c, c->stream, nullptr);
+    long lead = 0;
+    {
+        long t = c->t, snap = c->t_snap;
+        for (; !(t % 10 == 0 && snap >= 0 && snap == t - 10) && t < t_end; ++t, ++lead)
+            if (t % 10 == 0) snap = t;
+    }
+    if (lead > 0) {
+        const glbe_status s = glbe_step_n(c, lead);
         if (s != GLBE_OK) return s;
     }
-    glbe_status s = build_chunk(c);
+    glbe_status s = GLBE_OK;
+    const bool resident = c->res.form != 0;
+    if (!resident) s = build_chunk(c);
     if (s != GLBE_OK) return s;
     misc_set_kernel<<<1, 1, 0, c->stream>>>(nullptr, 0, c->stop_dev, 0, c->tol_dev, tol, nullptr, nullptr, 0);
     GLBE_CUDA(cudaGetLastError(), "solve setup");
-    const long batch = 16;       // chunks between host checks
+    // chunks between host checks: a resident march ends by itself when it
+    // converges, so its launches can be long
+    const long batch = resident ? 512 : 16;
     int stop = 0;
     while (c->t + 10 <= t_end) {
         long nb = 0;
         for (; nb < batch && c->t + 10 * (nb + 1) <= t_end; ++nb)
-            GLBE_CUDA(cudaGraphLaunch(c->chunk, c->stream), "graph launch");
-        GLBE_CUDA(cudaStreamSynchronize(c->stream), "solve sync");
-        GLBE_CUDA(cudaMemcpy(&stop, c->stop_dev, sizeof(int), cudaMemcpyDeviceToHost), "solve read");
+            if (!resident) GLBE_CUDA(cudaGraphLaunch(c->chunk, c->stream), "graph launch");
+        if (resident) {
+            s = enqueue_resident(c, 10 * nb, true, tol);
+            if (s != GLBE_OK) return s;
+        }
+        s = sync_control(c, &stop);
+        if (s != GLBE_OK) return s;
         if (stop) {
             glbe_residual_info info;
             glbe_status rs = read_record(c, &info);
@@ -786,12 +890,14 @@ glbe_status glbe_solve(glbe_ctx* c, double tol, long max_steps, long* steps_out,
             GLBE_CUDA(cudaGetLastError(), "solve reset");
             return rs;
         }
-        c->t += 10 * nb;
-        c->t_snap = c->t - 10;
+        if (!resident) {
+            c->t += 10 * nb;
+            c->t_snap = c->t - 10;
+        }
     }
     // finish with plain steps if max_steps is not a multiple of 10
-    while (c->t < t_end) {
-        s = enqueue_step(c, c->stream, nullptr);
+    if (c->t < t_end) {
+        s = glbe_step_n(c, t_end - c->t);
         if (s != GLBE_OK) return s;
     }
     glbe_residual_info info;

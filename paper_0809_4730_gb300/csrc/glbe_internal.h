@@ -167,6 +167,51 @@ cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, lo
                             double* record, double* hist, unsigned long long* hist_count, unsigned hist_cap,
                             int* stop, const double* tol, cudaStream_t st);
 
+// Where a residual evaluation is recorded.
+struct RecordOut {
+    double* record;                    // RECORD_STRIDE values
+    double* hist;                      // ring of hist_cap records
+    unsigned long long* hist_count;
+    unsigned hist_cap;
+    long long* t_dev;                  // level of the next residual evaluation
+    int* stop;                         // raised when r <= *tol or a velocity is not finite
+    const double* tol;
+    double mass0;
+};
+
+// One launch of a resident march (glbe_resident.cuh): levels t0 .. t0 + nsteps
+// - 1 are collided.  solve: the march ends at the first residual level with
+// r <= tol or a non-finite velocity (and does nothing if *out.stop is set on
+// entry); otherwise it takes every step, as single steps do.
+struct ResidentMarch {
+    void* f[2];
+    void* g[2];
+    float* FL;
+    const float* Ffield;
+    float* usnap;
+    double* partials;
+    int snap_lo;
+    int have_snap;        // the snapshot is of the residual level before the first one of this march
+    long long t0, nsteps;
+    int solve;
+    double tol;
+    RecordOut out;
+    unsigned* bar;        // barrier count, barrier generation, error flag
+};
+
+// How a grid's resident march is launched; form 0: it is not.
+struct ResidentPlan {
+    int form;             // 1 one cluster, 2 one tile a block, 3 dense (several tiles a block)
+    int pair;             // two nodes per thread
+    int blocks, threads;
+    unsigned smem;
+};
+template <int ST>
+cudaError_t resident_plan(bool mhd, const StepParams& p, ResidentPlan* out);
+template <int ST>
+cudaError_t resident_march(bool mhd, const StepParams& p, const ResidentMarch& m, const ResidentPlan& pl,
+                           cudaStream_t st);
+
 // Host helpers shared by the C-ABI translation units (glbe_api.cu).
 glbe_status fail(glbe_status s, const char* fmt, ...);       // sets the thread-local message
 glbe_status validate_params(const glbe_params* p);

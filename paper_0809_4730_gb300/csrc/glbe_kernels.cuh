@@ -50,7 +50,31 @@ __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, 
 __device__ __forceinline__ F2 operator-(F2 a) { return F2(__fmul2_rn(a.v, make_float2(-1.f, -1.f))); }
 __device__ __forceinline__ F2& operator+=(F2& a, F2 b) { a = a + b; return a; }
 
+// One node in F2's arithmetic: both lanes hold it, so a node updated alone
+// gives the bits that it gives as half of a pair.  (Scalar __fadd_rn /
+// __fmul_rn in the same places do not: the packed operations' roundings are
+// not all theirs.)
+struct F1 {
+    F2 w;
+    __device__ __forceinline__ F1() {}
+    __device__ __forceinline__ explicit F1(float c) : w(c) {}
+    __device__ __forceinline__ explicit F1(F2 c) : w(c) {}
+    __device__ __forceinline__ float lane() const { return w.v.x; }
+};
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return F1(a.w + b.w); }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return F1(a.w - b.w); }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return F1(a.w * b.w); }
+__device__ __forceinline__ F1 operator-(F1 a) { return F1(-a.w); }
+__device__ __forceinline__ F1& operator+=(F1& a, F1 b) { a = a + b; return a; }
+
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+// FP32 values of the one or two nodes of a V
+__device__ __forceinline__ void ldv(const float* p, F1& v) { v = F1(*p); }
+__device__ __forceinline__ void ldv(const float* p, F2& v) { v = F2(*reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ void ldgv(const float* p, F1& v) { v = F1(__ldg(p)); }
+__device__ __forceinline__ void ldgv(const float* p, F2& v) { v = F2(__ldg(reinterpret_cast<const float2*>(p))); }
+__device__ __forceinline__ void stv(float* p, F1 v) { *p = v.lane(); }
+__device__ __forceinline__ void stv(float* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 // additions/subtractions that must not be contracted or reassociated
 __device__ __forceinline__ float vadd_rn(float a, float b) { return __fadd_rn(a, b); }
@@ -63,6 +87,12 @@ __device__ __forceinline__ float lane_sum(float a) { return a; }
 __device__ __forceinline__ float lane_sum(F2 a) { return a.v.x + a.v.y; }
 __device__ __forceinline__ float vnonfinite(float a) { return isfinite(a) ? 0.f : 1.f; }
 __device__ __forceinline__ float vnonfinite(F2 a) { return (isfinite(a.v.x) ? 0.f : 1.f) + (isfinite(a.v.y) ? 0.f : 1.f); }
+__device__ __forceinline__ F1 vfma(F1 a, F1 b, F1 c) { return F1(vfma(a.w, b.w, c.w)); }
+__device__ __forceinline__ F1 vadd_rn(F1 a, F1 b) { return a + b; }
+__device__ __forceinline__ F1 vsub_rn(F1 a, F1 b) { return a - b; }
+__device__ __forceinline__ F1 vrcp(F1 a) { return F1(1.0f / a.lane()); }
+__device__ __forceinline__ float lane_sum(F1 a) { return a.lane(); }
+__device__ __forceinline__ float vnonfinite(F1 a) { return isfinite(a.lane()) ? 0.f : 1.f; }
 
 // fl(a + b + c) for |c| small: the exact two-sum of a and b, its remainder
 // plus c, rounded once.
@@ -290,6 +320,12 @@ __device__ __forceinline__ void store_pair(typename Store<ST>::T* p, F2 v, SrBit
     else Store<ST>::st2(p, v);
 }
 
+template <int ST>
+__device__ __forceinline__ void store_pair(typename Store<ST>::T* p, F1 v, SrBits& rb)
+{
+    *p = store_cv<ST>(v.lane(), rb);
+}
+
 // Loads of populations written earlier in the same launch (the persistent
 // batch kernel) must not use the non-coherent read-only path.  CG = true
 // gathers with coherent loads that are still cached in L1 (ld.global.ca):
@@ -317,6 +353,10 @@ __device__ __forceinline__ float ldlo(const __half* p)
 
 template <int ST>
 __device__ __forceinline__ float unscale(const StepParams& p, float v) { return Store<ST>::SCALED ? v * p.inv_scale : v; }
+template <int ST>
+__device__ __forceinline__ F1 unscale(const StepParams& p, F1 v) { return Store<ST>::SCALED ? v * F1(p.inv_scale) : v; }
+template <int ST>
+__device__ __forceinline__ F1 toscale(const StepParams& p, F1 v) { return Store<ST>::SCALED ? v * F1(p.scale) : v; }
 template <int ST>
 __device__ __forceinline__ F2 unscale(const StepParams& p, F2 v) { return Store<ST>::SCALED ? v * F2(p.inv_scale) : v; }
 template <int ST>
@@ -1281,35 +1321,41 @@ __device__ __forceinline__ NodeIn<float> node_inputs(const StepParams& p, const 
     return in;
 }
 
-template <bool MHD, int MODE>
-__device__ __forceinline__ NodeIn<F2> pair_inputs(const StepParams& p, const StepBuffers& b, uint32_t n0)
+template <bool MHD, int MODE, class V = F2>
+__device__ __forceinline__ NodeIn<V> pair_inputs(const StepParams& p, const StepBuffers& b, uint32_t n0)
 {
     const size_t N = p.N;
-    NodeIn<F2> in;
-    in.FLx = in.FLy = in.FLz = F2(0.f);
+    NodeIn<V> in;
+    in.FLx = in.FLy = in.FLz = V(0.f);
     if (MHD) {
-        in.FLx = F2(*reinterpret_cast<const float2*>(b.FL + n0));
-        in.FLy = F2(*reinterpret_cast<const float2*>(b.FL + N + n0));
-        in.FLz = F2(*reinterpret_cast<const float2*>(b.FL + 2 * N + n0));
+        ldv(b.FL + n0, in.FLx);
+        ldv(b.FL + N + n0, in.FLy);
+        ldv(b.FL + 2 * N + n0, in.FLz);
     }
-    in.Fx = F2(p.F[0]);
-    in.Fy = F2(p.F[1]);
-    in.Fz = F2(p.F[2]);
-    if (p.force_ncomp >= 1) in.Fx += F2(__ldg(reinterpret_cast<const float2*>(b.Ffield + n0)));
+    in.Fx = V(p.F[0]);
+    in.Fy = V(p.F[1]);
+    in.Fz = V(p.F[2]);
+    V v;
+    if (p.force_ncomp >= 1) {
+        ldgv(b.Ffield + n0, v);
+        in.Fx += v;
+    }
     if (p.force_ncomp == 3) {
-        in.Fy += F2(__ldg(reinterpret_cast<const float2*>(b.Ffield + N + n0)));
-        in.Fz += F2(__ldg(reinterpret_cast<const float2*>(b.Ffield + 2 * N + n0)));
+        ldgv(b.Ffield + N + n0, v);
+        in.Fy += v;
+        ldgv(b.Ffield + 2 * N + n0, v);
+        in.Fz += v;
     }
-    in.us0 = in.us1 = in.us2 = F2(0.f);
-    in.ul0 = in.ul1 = in.ul2 = F2(0.f);
+    in.us0 = in.us1 = in.us2 = V(0.f);
+    in.ul0 = in.ul1 = in.ul2 = V(0.f);
     if (MODE == MODE_STEP_RESID && b.have_snap) {
-        in.us0 = F2(*reinterpret_cast<const float2*>(b.usnap + n0));
-        in.us1 = F2(*reinterpret_cast<const float2*>(b.usnap + N + n0));
-        in.us2 = F2(*reinterpret_cast<const float2*>(b.usnap + 2 * N + n0));
+        ldv(b.usnap + n0, in.us0);
+        ldv(b.usnap + N + n0, in.us1);
+        ldv(b.usnap + 2 * N + n0, in.us2);
         if (b.snap_lo) {
-            in.ul0 = F2(*reinterpret_cast<const float2*>(b.usnap + 3 * N + n0));
-            in.ul1 = F2(*reinterpret_cast<const float2*>(b.usnap + 4 * N + n0));
-            in.ul2 = F2(*reinterpret_cast<const float2*>(b.usnap + 5 * N + n0));
+            ldv(b.usnap + 3 * N + n0, in.ul0);
+            ldv(b.usnap + 4 * N + n0, in.ul1);
+            ldv(b.usnap + 5 * N + n0, in.ul2);
         }
     }
     return in;
@@ -1732,19 +1778,20 @@ __global__ void __launch_bounds__(STEP_THREADS, ST == ST_F32C ? 2 : 3)
 
 // The update of the fluid node pair (n0, n0 + 1) from its gathered
 // pre-collision populations (packed FP32x2): the counterpart of
-// node_from_sources for two nodes; adds the pair's residual terms to acc.
+// node_from_sources for two nodes (V = F1: for the one node n0, in the same
+// arithmetic); adds the pair's residual terms to acc.
 // DIR: the f stores address the per-direction bases b.fdst_dir.
-template <int ST, bool MHD, int MODE, bool DIR = false>
+template <int ST, bool MHD, int MODE, bool DIR = false, class V = F2>
 __device__ __forceinline__ void pair_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n0,
-                                                  const F2 (&d)[19], const F2 (&dl)[19], const F2 (&q)[21],
-                                                  const F2 (&ql)[21], const NodeIn<F2>& in, float (&acc)[7])
+                                                  const V (&d)[19], const V (&dl)[19], const V (&q)[21],
+                                                  const V (&ql)[21], const NodeIn<V>& in, float (&acc)[7])
 {
     using S = Store<ST>;
     using T = typename S::T;
     const size_t N = p.N;
-    F2 om[19], og[21];
-    NodeState<F2> ns;
-    node_update<F2, ST, MHD>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz, true, om, og, ns);
+    V om[19], og[21];
+    NodeState<V> ns;
+    node_update<V, ST, MHD>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz, true, om, og, ns);
 
     T* __restrict__ fd = static_cast<T*>(b.fdst);
     [[maybe_unused]] SrBits rb(n0, step_seed<ST>(b));
@@ -1752,7 +1799,7 @@ __device__ __forceinline__ void pair_from_sources(const StepParams& p, const Ste
         __half* __restrict__ fdl = reinterpret_cast<__half*>(fd + 19 * N);
 #pragma unroll
         for (int a = 0; a < 19; ++a) {
-            F2 nh, nl;
+            V nh, nl;
             comp_add(d[a], dl[a], om[a], nh, nl);
             S::st2(fd + (size_t)a * N + n0, nh);
             S::st2_lo(fdl + (size_t)a * N + n0, nl);
@@ -1772,7 +1819,7 @@ __device__ __forceinline__ void pair_from_sources(const StepParams& p, const Ste
             __half* __restrict__ gdl = reinterpret_cast<__half*>(gd + 21 * N);
 #pragma unroll
             for (int a = 0; a < 21; ++a) {
-                F2 nh, nl;
+                V nh, nl;
                 comp_add(q[a], ql[a], og[a], nh, nl);
                 S::st2(gd + (size_t)a * N + n0, nh);
                 S::st2_lo(gdl + (size_t)a * N + n0, nl);
@@ -1781,18 +1828,15 @@ __device__ __forceinline__ void pair_from_sources(const StepParams& p, const Ste
 #pragma unroll
             for (int a = 0; a < 21; ++a) store_pair<ST>(gd + (size_t)a * N + n0, toscale<ST>(p, q[a] + og[a]), rb);
         }
-        *reinterpret_cast<float2*>(b.FL + n0) = ns.mac.FLx.v;
-        *reinterpret_cast<float2*>(b.FL + N + n0) = ns.mac.FLy.v;
-        *reinterpret_cast<float2*>(b.FL + 2 * N + n0) = ns.mac.FLz.v;
+        stv(b.FL + n0, ns.mac.FLx);
+        stv(b.FL + N + n0, ns.mac.FLy);
+        stv(b.FL + 2 * N + n0, ns.mac.FLz);
     }
     if (MODE == MODE_STEP_RESID) {
-        float2* us = reinterpret_cast<float2*>(b.usnap + n0);
-        float2* vs = reinterpret_cast<float2*>(b.usnap + N + n0);
-        float2* ws = reinterpret_cast<float2*>(b.usnap + 2 * N + n0);
         if (b.have_snap) {
-            const F2 dx = (ns.ux - in.us0) + (ns.ulx - in.ul0);
-            const F2 dy = (ns.uy - in.us1) + (ns.uly - in.ul1);
-            const F2 dz = (ns.uz - in.us2) + (ns.ulz - in.ul2);
+            const V dx = (ns.ux - in.us0) + (ns.ulx - in.ul0);
+            const V dy = (ns.uy - in.us1) + (ns.uly - in.ul1);
+            const V dz = (ns.uz - in.us2) + (ns.ulz - in.ul2);
             acc[0] += lane_sum(dx * dx + dy * dy + dz * dz);
         }
         acc[1] += lane_sum(ns.ux * ns.ux + ns.uy * ns.uy + ns.uz * ns.uz);
@@ -1801,13 +1845,13 @@ __device__ __forceinline__ void pair_from_sources(const StepParams& p, const Ste
         acc[4] += lane_sum(ns.jy);
         acc[5] += lane_sum(ns.jz);
         acc[6] += vnonfinite(ns.ux + ns.uy + ns.uz);
-        *us = ns.ux.v;
-        *vs = ns.uy.v;
-        *ws = ns.uz.v;
+        stv(b.usnap + n0, ns.ux);
+        stv(b.usnap + N + n0, ns.uy);
+        stv(b.usnap + 2 * N + n0, ns.uz);
         if (b.snap_lo) {
-            *reinterpret_cast<float2*>(b.usnap + 3 * N + n0) = ns.ulx.v;
-            *reinterpret_cast<float2*>(b.usnap + 4 * N + n0) = ns.uly.v;
-            *reinterpret_cast<float2*>(b.usnap + 5 * N + n0) = ns.ulz.v;
+            stv(b.usnap + 3 * N + n0, ns.ulx);
+            stv(b.usnap + 4 * N + n0, ns.uly);
+            stv(b.usnap + 5 * N + n0, ns.ulz);
         }
     }
 }

@@ -38,17 +38,15 @@ __device__ __forceinline__ double partial_row_sum(const double* row, unsigned b0
     return t;
 }
 
-// Where a residual evaluation is recorded.
-struct RecordOut {
-    double* record;                    // RECORD_STRIDE values
-    double* hist;                      // ring of hist_cap records
-    unsigned long long* hist_count;
-    unsigned hist_cap;
-    long long* t_dev;                  // level of the next residual evaluation
-    int* stop;                         // raised when r <= *tol or a velocity is not finite
-    const double* tol;
-    double mass0;
-};
+// The same of at most 32 values in shared memory.
+__device__ __forceinline__ double partial_row_sum_shared(const double* row, int n)
+{
+    const int lane = threadIdx.x & 31;
+    double t = lane < n ? row[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
 
 // r(t) of the sums (Sec. 5): ||u(t) - u(t-10)|| / ||u(t)||.
 __device__ __forceinline__ double residual_of(double num, double den)

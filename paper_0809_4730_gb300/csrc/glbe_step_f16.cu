@@ -2,6 +2,7 @@
 // population deviations (one translation unit per storage type so they
 // compile in parallel).
 #include "glbe_kernels.cuh"
+#include "glbe_resident.cuh"
 
 namespace glbe {
 template cudaError_t launch_step_t<ST_F16>(bool, int, const StepParams&, const StepBuffers&, const FieldOut&,
@@ -11,4 +12,7 @@ template cudaError_t launch_get_state_t<ST_F16>(bool, const StepParams&, const v
 template cudaError_t launch_set_state_t<ST_F16>(bool, const StepParams&, void*, void*, float*, const float*,
                                                 const float*, const float*, cudaStream_t);
 template int tile_wait_error_t<ST_F16>();
+template cudaError_t resident_plan<ST_F16>(bool, const StepParams&, ResidentPlan*);
+template cudaError_t resident_march<ST_F16>(bool, const StepParams&, const ResidentMarch&, const ResidentPlan&,
+                                          cudaStream_t);
 }  // namespace glbe

@@ -2,6 +2,7 @@
 // population deviations (one translation unit per storage type so they
 // compile in parallel).
 #include "glbe_kernels.cuh"
+#include "glbe_resident.cuh"
 
 namespace glbe {
 template cudaError_t launch_step_t<ST_F32>(bool, int, const StepParams&, const StepBuffers&, const FieldOut&,
@@ -12,4 +13,7 @@ template cudaError_t launch_set_state_t<ST_F32>(bool, const StepParams&, void*, 
                                                 const float*, const float*, cudaStream_t);
 template int tile_wait_error_t<ST_F32>();
 template cudaError_t launch_lid_init_t<ST_F32>(const StepParams&, void*, cudaStream_t);
+template cudaError_t resident_plan<ST_F32>(bool, const StepParams&, ResidentPlan*);
+template cudaError_t resident_march<ST_F32>(bool, const StepParams&, const ResidentMarch&, const ResidentPlan&,
+                                          cudaStream_t);
 }  // namespace glbe
