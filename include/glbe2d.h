@@ -109,7 +109,8 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
 glbe_status glbe2d_set_force(glbe2d_ctx* ctx, const float* d_F);
 
 /* Advances n >= 0 steps; the step colliding a level t with t % 10 == 0 also
- * evaluates the residual. */
+ * evaluates the residual.  With the automatic kernel form, small grids (up to
+ * about 600,000 nodes) take n >= 2 steps in one launch, as in glbe_step_n. */
 glbe_status glbe2d_step_n(glbe2d_ctx* ctx, long n);
 
 /* Synchronises and returns the latest residual record (momentum[2] = 0).
@@ -121,7 +122,7 @@ glbe_status glbe2d_history(glbe2d_ctx* ctx, glbe_residual_info* out, long cap, l
 
 /* Marches until r(t) <= tol at a level t that is a multiple of 10, or until
  * max_steps steps were taken, replaying a CUDA graph of 10-step chunks whose
- * kernels stop on a device flag.  *steps_out = the converged level (or the
+ * kernels stop on a device flag (small grids: resident launches).  *steps_out = the converged level (or the
  * level reached), *r_out = its r.  GLBE_ERR_TIMEOUT / GLBE_ERR_DIVERGED as
  * glbe_solve.  Syncs. */
 glbe_status glbe2d_solve(glbe2d_ctx* ctx, double tol, long max_steps, long* steps_out, double* r_out);

@@ -32,6 +32,7 @@
 
 #include "glbe2d.h"
 #include "glbe_internal.h"
+#include "glbe_resident_common.cuh"
 
 using namespace glbe;
 
@@ -805,6 +806,73 @@ __device__ __forceinline__ void prefetch2d(const P2& p, const B2& b)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((uint32_t)(hi - lo)) : "memory");
 }
 
+// The update of fluid node n from its gathered populations: fields (M2_FIELDS)
+// or the collision and the stores into its own slots of the other buffer;
+// residual levels add to acc.
+template <int ST, bool MHD, int MODE>
+__device__ __forceinline__ void node2_from_sources(const P2& p, const B2& b, const Out2& o, int n, const float (&d)[9],
+                                                   const float (&dl)[9], const float (&q)[10], const float (&ql)[10],
+                                                   float (&us)[4], float (&acc)[7])
+{
+    float Fex = p.Fx, Fey = p.Fy;
+    if (b.Ffield) {
+        Fex += __ldg(b.Ffield + n);
+        Fey += __ldg(b.Ffield + p.N + n);
+    }
+    const float FLpx = MHD ? b.FL[n] : 0.f, FLpy = MHD ? b.FL[p.N + n] : 0.f;
+    Node2 nd;
+    float Fx, Fy, om[9], og[10];
+    if constexpr (ST == GLBE_BF16) {
+        Node2V<float> v;
+        node_update2v<float, MHD, MODE != M2_FIELDS>(p, d, q, Fex, Fey, FLpx, FLpy, v, Fx, Fy, om, og);
+        nd = Node2{v.rho, v.jx, v.jy, v.ux, v.uy, v.Bx, v.By, v.FLx, v.FLy};
+    } else {
+        node_update2<ST, MHD, MODE != M2_FIELDS>(p, d, dl, q, ql, Fex, Fey, FLpx, FLpy, nd, Fx, Fy, om, og);
+    }
+    if constexpr (MODE == M2_FIELDS) {
+        if (o.rho) o.rho[n] = nd.rho;
+        if (o.u) {
+            o.u[n] = nd.ux;
+            o.u[p.N + n] = nd.uy;
+        }
+        if (MHD && o.B) {
+            o.B[n] = nd.Bx;
+            o.B[p.N + n] = nd.By;
+        }
+    } else {
+        const size_t N = p.N;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) put<ST>(b.fdst, N, 9, (size_t)a * N + n, d[a], dl[a], om[a]);
+        if (MHD) {
+#pragma unroll
+            for (int i = 0; i < 10; ++i) put<ST>(b.gdst, N, 10, (size_t)i * N + n, q[i], ql[i], og[i]);
+            b.FL[n] = nd.FLx;
+            b.FL[N + n] = nd.FLy;
+        }
+        if constexpr (MODE == M2_RESID) {
+            resid_node(p, d, dl, Fx, Fy, b.have_snap, us, acc);
+            b.usnap[n] = us[0];
+            b.usnap[N + n] = us[1];
+            b.usnap[2 * N + n] = us[2];
+            b.usnap[3 * N + n] = us[3];
+        }
+    }
+}
+
+// The residual snapshot of node n: read before the node's stores, since a load
+// after them waits for them (the stores may alias it).
+template <int MODE>
+__device__ __forceinline__ void load_snap2(const P2& p, const B2& b, int n, float (&us)[4])
+{
+    us[0] = us[1] = us[2] = us[3] = 0.f;
+    if (MODE == M2_RESID && b.have_snap) {
+        us[0] = b.usnap[n];
+        us[1] = b.usnap[p.N + n];
+        us[2] = b.usnap[2 * (size_t)p.N + n];
+        us[3] = b.usnap[3 * (size_t)p.N + n];
+    }
+}
+
 // One node per thread: any geometry.
 template <int ST, bool MHD, int MODE>
 __device__ __forceinline__ void step2d_body(const P2& p, const B2& b, const Out2& o)
@@ -821,15 +889,8 @@ __device__ __forceinline__ void step2d_body(const P2& p, const B2& b, const Out2
             if (o.u) o.u[n] = o.u[p.N + n] = 0.f;
             if (MHD && o.B) o.B[n] = o.B[p.N + n] = 0.f;
         } else if (!is_solid(p, x, y)) {
-            // the residual snapshot is read before the node's stores: a load
-            // after them waits for them (the stores may alias it)
-            float us[4] = {0.f, 0.f, 0.f, 0.f};
-            if (MODE == M2_RESID && b.have_snap) {
-                us[0] = b.usnap[n];
-                us[1] = b.usnap[p.N + n];
-                us[2] = b.usnap[2 * (size_t)p.N + n];
-                us[3] = b.usnap[3 * (size_t)p.N + n];
-            }
+            float us[4];
+            load_snap2<MODE>(p, b, n, us);
             float d[9], dl[9], q[10], ql[10];
             if (x >= p.ix0 && x <= p.ix1 && y >= p.iy0 && y <= p.iy1) {
                 gather_f_interior<ST>(p, n, b.fsrc, d, dl);
@@ -839,49 +900,7 @@ __device__ __forceinline__ void step2d_body(const P2& p, const B2& b, const Out2
                 gather_f<ST>(p, nb, x, y, n, b.fsrc, d, dl);
                 if (MHD) gather_g<ST>(p, nb, x, y, n, b.gsrc, q, ql);
             }
-            float Fex = p.Fx, Fey = p.Fy;
-            if (b.Ffield) {
-                Fex += __ldg(b.Ffield + n);
-                Fey += __ldg(b.Ffield + p.N + n);
-            }
-            const float FLpx = MHD ? b.FL[n] : 0.f, FLpy = MHD ? b.FL[p.N + n] : 0.f;
-            Node2 nd;
-            float Fx, Fy, om[9], og[10];
-            if constexpr (ST == GLBE_BF16) {
-                Node2V<float> v;
-                node_update2v<float, MHD, MODE != M2_FIELDS>(p, d, q, Fex, Fey, FLpx, FLpy, v, Fx, Fy, om, og);
-                nd = Node2{v.rho, v.jx, v.jy, v.ux, v.uy, v.Bx, v.By, v.FLx, v.FLy};
-            } else {
-                node_update2<ST, MHD, MODE != M2_FIELDS>(p, d, dl, q, ql, Fex, Fey, FLpx, FLpy, nd, Fx, Fy, om, og);
-            }
-            if constexpr (MODE == M2_FIELDS) {
-                if (o.rho) o.rho[n] = nd.rho;
-                if (o.u) {
-                    o.u[n] = nd.ux;
-                    o.u[p.N + n] = nd.uy;
-                }
-                if (MHD && o.B) {
-                    o.B[n] = nd.Bx;
-                    o.B[p.N + n] = nd.By;
-                }
-            } else {
-                const size_t N = p.N;
-#pragma unroll
-                for (int a = 0; a < 9; ++a) put<ST>(b.fdst, N, 9, (size_t)a * N + n, d[a], dl[a], om[a]);
-                if (MHD) {
-#pragma unroll
-                    for (int i = 0; i < 10; ++i) put<ST>(b.gdst, N, 10, (size_t)i * N + n, q[i], ql[i], og[i]);
-                    b.FL[n] = nd.FLx;
-                    b.FL[N + n] = nd.FLy;
-                }
-                if constexpr (MODE == M2_RESID) {
-                    resid_node(p, d, dl, Fx, Fy, b.have_snap, us, acc);
-                    b.usnap[n] = us[0];
-                    b.usnap[N + n] = us[1];
-                    b.usnap[2 * N + n] = us[2];
-                    b.usnap[3 * N + n] = us[3];
-                }
-            }
+            node2_from_sources<ST, MHD, MODE>(p, b, o, n, d, dl, q, ql, us, acc);
         }
     }
     if constexpr (MODE == M2_RESID) block_partials2(acc, b.partials);
@@ -917,6 +936,253 @@ template <int ST, bool MHD>
 constexpr int dense2d_blocks()
 {
     return ST == GLBE_F32 ? (MHD ? 4 : 6) : (ST == GLBE_BF16 ? (MHD ? 0 : 8) : (MHD ? 3 : 5));
+}
+
+// ---------------------------------------------------------------------------
+// Resident march of small grids (glbe_resident_common.cuh): many steps in one
+// launch, one node per thread, the one-node kernel's arithmetic bit for bit.
+// Table rows: the source node of each D2Q9 direction (the node itself where
+// the link is bounced) and the bounced-link bits; the D2Q5 directions share
+// the sources of the axis directions.  A step takes (us, launched -> resident):
+//               F32 flow      F32 coupled   F32C coupled  BF16 coupled
+//   64 x 64     6.4 -> 1.7    6.6 -> 2.3    8.6 -> 3.0    6.7 -> 2.2
+//   128 x 128   6.5 -> 2.8    6.6 -> 3.5    8.5 -> 4.0    6.6 -> 3.2
+//   384 x 384   8.7 -> 5.9    8.9 -> 7.0   13.0 -> 10.9   8.9 -> 6.1
+// The line lies where the tables crowd out the gathers' L1: 820 x 820 coupled
+// F32 marched 29.5 us a step with 205 KB of tables on an SM and 24.3 launched,
+// 700 x 700 18.1 with 164 KB and 18.4 launched.
+// ---------------------------------------------------------------------------
+constexpr int RES2_ROWS = 10;
+constexpr size_t RES2_TABLES = (size_t)16 * RES2_ROWS * 256 * 4;   // table bytes of an SM, at most
+__host__ __device__ constexpr int axis9(int a5) { return a5 == 0 ? 0 : (a5 == 1 ? 1 : (a5 == 2 ? 3 : (a5 == 3 ? 2 : 4))); }
+static_assert(ex9(axis9(2)) == ex5(2) && ey9(axis9(3)) == ey5(3), "D2Q5 directions among the D2Q9 ones");
+
+__device__ __forceinline__ void resident_slots2(const P2& p, uint32_t i, uint32_t* tab, int stride)
+{
+    tab[9 * stride] = RES_SKIP;
+    if (i >= (uint32_t)p.N) return;
+    const int n = (int)i, y = row_of(p, n), x = n - y * p.nx;
+    if (is_solid(p, x, y)) return;
+    const Nb nb = neighbours(p, x, y);
+    unsigned bounced = 0;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        bool sol;
+        const int s = source(p, nb, x, y, ex9(a), ey9(a), sol);
+        tab[a * stride] = (uint32_t)(sol ? n : s);
+        bounced |= sol ? 1u << a : 0u;
+    }
+    tab[9 * stride] = bounced;
+}
+
+// Coherent loads, cached in L1 within a level (the non-coherent path must not
+// serve populations written earlier in the launch).
+__device__ __forceinline__ float ldca2(const float* p) { return __ldca(p); }
+__device__ __forceinline__ float ldca2(const __nv_bfloat16* p)
+{
+    return __uint_as_float((unsigned)__ldca(reinterpret_cast<const unsigned short*>(p)) << 16);
+}
+__device__ __forceinline__ float ldca2_lo(const __half* p) { return __half2float(__ldca(p)) * LO2_INV; }
+
+template <int ST, bool MHD, int MODE>
+__device__ __forceinline__ void resident_update2(const P2& p, const B2& b, int n, const uint32_t* tab, int stride,
+                                                 unsigned bounced, float (&acc)[7])
+{
+    using S = Sto2<ST>;
+    using T = typename S::T;
+    const size_t N = p.N;
+    float us[4], d[9], dl[9], q[10], ql[10];
+    load_snap2<MODE>(p, b, n, us);
+    const T* f = static_cast<const T*>(b.fsrc);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        const size_t k = ((bounced >> a) & 1u ? (size_t)opp9t(a) : (size_t)a) * N + tab[a * stride];
+        d[a] = ldca2(f + k);
+        dl[a] = S::COMP ? ldca2_lo(reinterpret_cast<const __half*>(f + 9 * N) + k) : 0.f;
+    }
+    if constexpr (MHD) {
+        const T* g = static_cast<const T*>(b.gsrc);
+#pragma unroll
+        for (int a = 0; a < 5; ++a) {
+            const bool back = (bounced >> axis9(a)) & 1u;
+            const size_t at = tab[axis9(a) * stride];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const size_t k = (size_t)(j * 5 + (back ? opp5(a) : a)) * N + at;
+                const float v = ldca2(g + k);
+                const float vl = S::COMP ? ldca2_lo(reinterpret_cast<const __half*>(g + 10 * N) + k) : 0.f;
+                q[j * 5 + a] = back ? -v : v;
+                ql[j * 5 + a] = back ? -vl : vl;
+            }
+        }
+    }
+    const Out2 o{nullptr, nullptr, nullptr};
+    node2_from_sources<ST, MHD, MODE>(p, b, o, n, d, dl, q, ql, us, acc);
+}
+
+// DENSE: several tiles a block, held to the register budgets of the launched
+// plain steps (BF16 coupled: free there, four blocks here).
+// Residual sums: a warp's FP32 sums, those of GROUP warps added in order (the
+// partial of a launched block), and from there on FP64: in the cluster form in
+// the launched reduction's order, in the others a block's partials first, so
+// that a level's sums are one number per block.
+template <int ST, bool MHD, bool DENSE, bool CLUSTER>
+__global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, MHD>() ? dense2d_blocks<ST, MHD>() : 4)
+    resident2d_kernel(const P2 p, const ResidentMarch m)
+{
+    constexpr int GROUP = T2D / 32;
+    extern __shared__ uint32_t slots[];          // [tile][RES2_ROWS][blockDim.x]
+    // warp sums: of the block's tile, or of the whole grid (CLUSTER)
+    __shared__ float wsum[RES_SUMS][CLUSTER ? RES_CLUSTER * RES_THREADS / 32 : RES_THREADS / 32];
+    __shared__ double bsum[RES_SUMS], tot[RES_SUMS];   // of the block's tiles; of the grid
+    __shared__ int verdict;
+    const int BT = blockDim.x, G = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = BT >> 5;
+    if (m.solve && *(volatile int*)m.out.stop) return;   // converged in an earlier launch
+    const uint32_t ntiles = ((uint32_t)p.N + BT - 1) / BT;
+    int mine = 0;
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, ++mine)
+        resident_slots2(p, tile * BT + threadIdx.x, slots + (size_t)mine * RES2_ROWS * BT + threadIdx.x, BT);
+    if constexpr (CLUSTER) {
+        for (int i = threadIdx.x; i < RES_SUMS * RES_CLUSTER * RES_THREADS / 32; i += BT) (&wsum[0][0])[i] = 0.f;
+        cluster_level_barrier();                 // every block's shared memory is there to write to
+    }
+    unsigned gen = 0;
+    if (!CLUSTER && threadIdx.x == 0) gen = *(volatile unsigned*)(m.bar + 1);
+    const bool writer = blockIdx.x == G - 1;    // the last block has no more tiles than any other
+    B2 b{};
+    b.FL = m.FL;
+    b.Ffield = m.Ffield;
+    b.usnap = m.usnap;
+    bool snap = m.have_snap != 0;               // the snapshot is of the previous residual level
+    int par = m.phase & 1;                      // t0 and t0 mod 10 have the same parity
+    for (int s = 0, phase = m.phase; s < m.nsteps; ++s, par ^= 1, phase = phase == 9 ? 0 : phase + 1) {
+        const bool resid = phase == 0;
+        b.fsrc = m.f[par];
+        b.fdst = m.f[par ^ 1];
+        b.gsrc = m.g[par];
+        b.gdst = m.g[par ^ 1];
+        b.have_snap = snap ? 1 : 0;
+        if (!CLUSTER && resid && threadIdx.x < RES_SUMS) bsum[threadIdx.x] = 0.0;
+        for (int k = 0; k < mine; ++k) {
+            const uint32_t tile = blockIdx.x + (uint32_t)k * G;
+            const uint32_t* tab = slots + (size_t)k * RES2_ROWS * BT + threadIdx.x;
+            const unsigned flags = tab[(RES2_ROWS - 1) * BT];
+            float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (!resid) {
+                if (flags != RES_SKIP)
+                    resident_update2<ST, MHD, M2_STEP>(p, b, (int)(tile * BT + threadIdx.x), tab, BT, flags, acc);
+            } else {
+                if (flags != RES_SKIP)
+                    resident_update2<ST, MHD, M2_RESID>(p, b, (int)(tile * BT + threadIdx.x), tab, BT, flags, acc);
+                if (!snap) continue;
+#pragma unroll
+                for (int r = 0; r < RES_SUMS; ++r) acc[r] = warp_sum(acc[r]);
+                if constexpr (CLUSTER) {
+                    // into every block's shared memory
+                    const int at = (int)tile * warps + warp;
+#pragma unroll
+                    for (int r = 0; r < RES_SUMS; ++r) acc[r] = __shfl_sync(0xffffffffu, acc[r], 0);
+                    if (lane < G) {
+                        auto cl = cooperative_groups::this_cluster();
+#pragma unroll
+                        for (int r = 0; r < RES_SUMS; ++r) *cl.map_shared_rank(&wsum[r][at], lane) = acc[r];
+                    }
+                } else {
+                    if (lane == 0) {
+#pragma unroll
+                        for (int r = 0; r < RES_SUMS; ++r) wsum[r][warp] = acc[r];
+                    }
+                    __syncthreads();
+                    if (threadIdx.x < RES_SUMS) {
+                        for (int q = 0; q < warps; q += GROUP) {
+                            float v = 0.f;
+#pragma unroll
+                            for (int w = 0; w < GROUP; ++w) v += wsum[threadIdx.x][q + w];
+                            bsum[threadIdx.x] += (double)v;
+                        }
+                    }
+                    __syncthreads();
+                }
+            }
+        }
+        const bool sums = resid && snap;
+        if constexpr (CLUSTER) {
+            cluster_level_barrier();
+            if (sums) {
+                for (int r = warp; r < RES_SUMS; r += warps) {
+                    double v = 0.0;
+                    if ((unsigned)lane * 32 * GROUP < (uint32_t)p.N) {
+                        float f = 0.f;
+#pragma unroll
+                        for (int w = 0; w < GROUP; ++w) f += wsum[r][lane * GROUP + w];
+                        v = (double)f;
+                    }
+                    v = warp_sum_all(v);
+                    if (lane == 0) tot[r] = v;
+                }
+            }
+        } else {
+            if (sums && threadIdx.x < RES_SUMS) m.partials[(size_t)threadIdx.x * G + blockIdx.x] = bsum[threadIdx.x];
+            if (!resident_barrier(m.bar, gen)) return;
+            if (sums && (m.solve || writer)) {
+                // a solve's blocks all take the decision (num, den, non-finite count), from the same numbers in
+                // the same order
+                const int rows = writer ? RES_SUMS : 3;
+                for (int j = warp; j < rows; j += warps) {
+                    const int r = !writer && j == 2 ? 6 : j;
+                    const double v = partial_row_sum(m.partials + (size_t)r * G, 0, (unsigned)G);
+                    if (lane == 0) tot[r] = v;
+                }
+            }
+        }
+        if (!resid) continue;
+        if (sums && (m.solve || writer)) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                verdict = m.solve && resident_stops(m.tol, tot);
+                if (writer && !*m.out.stop) write_record(m.out, tot, *m.out.t_dev);
+            }
+            __syncthreads();
+            if (verdict) return;                // the state is the one after level t, in every block
+        }
+        if (!snap && writer && threadIdx.x == 0) *m.out.t_dev = m.t0 + s + 10;
+        snap = true;
+    }
+}
+
+template <int ST, bool MHD>
+cudaError_t resident2d_plan_t(uint32_t N, ResidentPlan* out)
+{
+    constexpr size_t tile = (size_t)RES2_ROWS * RES_THREADS * sizeof(uint32_t);
+    auto* cluster = resident2d_kernel<ST, MHD, false, true>;
+    auto* free_form = resident2d_kernel<ST, MHD, false, false>;
+    auto* dense = resident2d_kernel<ST, MHD, true, false>;
+    static const ResidentOcc of = resident_occupancy(free_form, tile), od = resident_occupancy(dense, tile);
+    static const bool fits = [&] {
+        cudaFuncSetAttribute(cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return resident_cluster_fits(cluster, tile);
+    }();
+    return resident_plan_of(cluster, free_form, dense, N, N, RES2_ROWS, RES2_TABLES, of, od, fits, out);
+}
+
+template <int ST>
+cudaError_t resident2d_plan(bool mhd, uint32_t N, ResidentPlan* out)
+{
+    return mhd ? resident2d_plan_t<ST, true>(N, out) : resident2d_plan_t<ST, false>(N, out);
+}
+
+template <int ST, bool MHD>
+cudaError_t resident2d_march_t(const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
+{
+    if (pl.form == 1) return resident_launch(resident2d_kernel<ST, MHD, false, true>, pl, st, p, m);
+    if (pl.form == 2) return resident_launch(resident2d_kernel<ST, MHD, false, false>, pl, st, p, m);
+    return resident_launch(resident2d_kernel<ST, MHD, true, false>, pl, st, p, m);
+}
+
+template <int ST>
+cudaError_t resident2d_march(bool mhd, const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
+{
+    return mhd ? resident2d_march_t<ST, true>(p, m, pl, st) : resident2d_march_t<ST, false>(p, m, pl, st);
 }
 
 // Two x-adjacent nodes per thread (x periodic, even nx; FP32 or BF16
@@ -1384,6 +1650,9 @@ struct glbe2d_ctx {
     cudaStream_t stream;
     cudaStream_t cap_stream;
     cudaGraphExec_t chunk;
+    unsigned* res_bar;      // barrier words of the resident march (count, generation, error)
+    ResidentPlan res;       // form 0: steps are launched one by one
+    bool res_used;          // a resident march was launched since the error flag was last read
 };
 
 namespace {
@@ -1527,10 +1796,87 @@ glbe_status enqueue2(glbe2d_ctx* c, cudaStream_t st, const int* stop)
     return GLBE_OK;
 }
 
+// The resident march serves the automatic kernel form.
+ResidentPlan plan_resident2(const glbe2d_ctx* c)
+{
+    ResidentPlan r{0, 0, 0, 0, 0};
+    if (c->prm.variant != 0 || c->N > RES_MAX_NODES) return r;
+    const bool mhd = c->prm.induction;
+    cudaError_t e;
+    switch (c->prm.storage) {
+    case GLBE_F32: e = resident2d_plan<GLBE_F32>(mhd, (uint32_t)c->N, &r); break;
+    case GLBE_BF16: e = resident2d_plan<GLBE_BF16>(mhd, (uint32_t)c->N, &r); break;
+    default: e = resident2d_plan<GLBE_F32C>(mhd, (uint32_t)c->N, &r); break;
+    }
+    if (e != cudaSuccess) {   // no plan: single launches, which report what is wrong
+        cudaGetLastError();
+        r.form = 0;
+    }
+    return r;
+}
+
+// Enqueues n >= 1 steps from level c->t as one resident march (solve: with the
+// stop test of tolerance tol).  The host's levels are those of a march that
+// takes every step.
+glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
+{
+    ResidentMarch m{};
+    for (int k = 0; k < 2; ++k) {
+        m.f[k] = c->f[k];
+        m.g[k] = c->prm.induction ? c->g[k] : nullptr;
+    }
+    m.FL = c->FL;
+    m.Ffield = c->Ffield;
+    m.usnap = c->usnap;
+    m.partials = c->partials;
+    const long first = (c->t + 9) / 10 * 10;        // first residual level of the march
+    m.have_snap = c->t_snap >= 0 && c->t_snap == first - 10;
+    m.t0 = c->t;
+    m.phase = (int)(c->t % 10);
+    m.nsteps = (int)n;
+    m.solve = solve ? 1 : 0;
+    m.tol = tol;
+    m.out = RecordOut{c->record, c->hist, c->hist_count, HIST_CAP2, c->t_dev, c->stop_dev, c->tol_dev, c->mass0};
+    m.bar = c->res_bar;
+    const bool mhd = c->prm.induction;
+    cudaError_t e;
+    switch (c->prm.storage) {
+    case GLBE_F32: e = resident2d_march<GLBE_F32>(mhd, c->p, m, c->res, c->stream); break;
+    case GLBE_BF16: e = resident2d_march<GLBE_BF16>(mhd, c->p, m, c->res, c->stream); break;
+    default: e = resident2d_march<GLBE_F32C>(mhd, c->p, m, c->res, c->stream); break;
+    }
+    GLBE2D_CUDA(e, "2D resident march");
+    c->res_used = true;
+    if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
+    c->t += n;
+    return GLBE_OK;
+}
+
+// Waits for the stream and reports whether a barrier wait of a resident march
+// ran out; stop (may be NULL) receives the march's stop flag.
+glbe_status sync_control2(glbe2d_ctx* c, int* stop)
+{
+    const bool resident = c->res_used && c->res.form >= 2;
+    c->res_used = false;
+    char* const base = reinterpret_cast<char*>(c->t_dev);   // start of the control words
+    char misc[64] = {0};
+    if (stop || resident)
+        GLBE2D_CUDA(cudaMemcpyAsync(misc, base, sizeof misc, cudaMemcpyDeviceToHost, c->stream), "2D control words");
+    GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D sync");
+    if (stop) std::memcpy(stop, misc + (reinterpret_cast<char*>(c->stop_dev) - base), sizeof *stop);
+    if (!resident) return GLBE_OK;
+    unsigned err = 0;
+    std::memcpy(&err, misc + (reinterpret_cast<char*>(c->res_bar + 2) - base), sizeof err);
+    if (!err) return GLBE_OK;
+    GLBE2D_CUDA(cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream), "2D resident march reset");
+    return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
+}
+
 glbe_status read_record2(glbe2d_ctx* c, glbe_residual_info* out)
 {
     double rec[RECORD_STRIDE];
-    GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D residual sync");
+    const glbe_status rs = sync_control2(c, nullptr);
+    if (rs != GLBE_OK) return rs;
     GLBE2D_CUDA(cudaMemcpy(rec, c->record, sizeof rec, cudaMemcpyDeviceToHost), "2D residual read");
     out->t = (long)rec[0];
     out->r = rec[1];
@@ -1648,12 +1994,16 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->hist_count = reinterpret_cast<unsigned long long*>(misc + 8);
     c->tol_dev = reinterpret_cast<double*>(misc + 16);
     c->stop_dev = reinterpret_cast<int*>(misc + 24);
+    c->res_bar = reinterpret_cast<unsigned*>(misc + 32);
+    c->res = plan_resident2(c);
+    c->res_used = false;
     c->mass0 = p->rho0 * (double)fluid2(p);
     c->t = 0;
     c->t_snap = -1;
     c->stream = static_cast<cudaStream_t>(p->stream);
     // the rest state: every deviation, the Lorentz force and the field zero
     cudaError_t e = cudaMemsetAsync(d_workspace, 0, L.record, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess) {
         ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record, c->hist_count, 1);
         e = cudaGetLastError();
@@ -1679,6 +2029,13 @@ glbe_status glbe2d_step_n(glbe2d_ctx* c, long n)
 {
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(GLBE_ERR_ARG, "n must be >= 0");
+    if (c->res.form && n >= 2) {
+        for (long k = 0; k < n; k += RES_MOST_STEPS) {
+            const glbe_status s = enqueue_resident2(c, n - k < RES_MOST_STEPS ? n - k : RES_MOST_STEPS, false, 0.0);
+            if (s != GLBE_OK) return s;
+        }
+        return GLBE_OK;
+    }
     for (long k = 0; k < n; ++k) {
         const glbe_status s = enqueue2(c, c->stream, nullptr);
         if (s != GLBE_OK) return s;
@@ -1728,24 +2085,32 @@ glbe_status glbe2d_solve(glbe2d_ctx* c, double tol, long max_steps, long* steps_
     if (!(tol > 0.0)) return fail(GLBE_ERR_ARG, "tol must be > 0");
     if (max_steps < 0) return fail(GLBE_ERR_ARG, "max_steps must be >= 0");
     const long t_end = c->t + max_steps;
-    while (!(c->t % 10 == 0 && c->t_snap >= 0 && c->t_snap == c->t - 10) && c->t < t_end) {
-        const glbe_status s = enqueue2(c, c->stream, nullptr);
-        if (s != GLBE_OK) return s;
-    }
-    glbe_status s = build_chunk2(c);
+    // up to a multiple of 10 with a snapshot at the one before
+    long lead = 0;
+    for (long t = c->t, snap = c->t_snap; !(t % 10 == 0 && snap >= 0 && snap == t - 10) && t < t_end; ++t, ++lead)
+        if (t % 10 == 0) snap = t;
+    glbe_status s = lead > 0 ? glbe2d_step_n(c, lead) : GLBE_OK;
+    if (s != GLBE_OK) return s;
+    const bool resident = c->res.form != 0;
+    if (!resident) s = build_chunk2(c);
     if (s != GLBE_OK) return s;
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(nullptr, 0, c->stop_dev, 0, c->tol_dev, tol, nullptr, nullptr, 0);
     GLBE2D_CUDA(cudaGetLastError(), "2D solve setup");
-    // chunks between host checks: about a millisecond of device work each
+    // chunks between host checks: about a millisecond of device work each (a
+    // resident march ends by itself when it converges)
     long batch = (long)(4000000 / (c->N + 1));
-    batch = batch < 4 ? 4 : (batch > 256 ? 256 : batch);
+    batch = resident ? 512 : batch < 4 ? 4 : (batch > 256 ? 256 : batch);
     int stop = 0;
     while (c->t + 10 <= t_end) {
         long nb = 0;
         for (; nb < batch && c->t + 10 * (nb + 1) <= t_end; ++nb)
-            GLBE2D_CUDA(cudaGraphLaunch(c->chunk, c->stream), "2D graph launch");
-        GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D solve sync");
-        GLBE2D_CUDA(cudaMemcpy(&stop, c->stop_dev, sizeof(int), cudaMemcpyDeviceToHost), "2D solve read");
+            if (!resident) GLBE2D_CUDA(cudaGraphLaunch(c->chunk, c->stream), "2D graph launch");
+        if (resident) {
+            s = enqueue_resident2(c, 10 * nb, true, tol);
+            if (s != GLBE_OK) return s;
+        }
+        s = sync_control2(c, &stop);
+        if (s != GLBE_OK) return s;
         if (stop) {
             glbe_residual_info info;
             const glbe_status rs = read_record2(c, &info);
@@ -1757,11 +2122,13 @@ glbe_status glbe2d_solve(glbe2d_ctx* c, double tol, long max_steps, long* steps_
             GLBE2D_CUDA(cudaGetLastError(), "2D solve reset");
             return rs;
         }
-        c->t += 10 * nb;
-        c->t_snap = c->t - 10;
+        if (!resident) {
+            c->t += 10 * nb;
+            c->t_snap = c->t - 10;
+        }
     }
-    while (c->t < t_end) {
-        s = enqueue2(c, c->stream, nullptr);
+    if (c->t < t_end) {
+        s = glbe2d_step_n(c, t_end - c->t);
         if (s != GLBE_OK) return s;
     }
     glbe_residual_info info;
@@ -1846,7 +2213,8 @@ glbe_status glbe2d_time(const glbe2d_ctx* c, long* t)
 glbe_status glbe2d_sync(glbe2d_ctx* c)
 {
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
-    GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D sync");
+    const glbe_status s = sync_control2(c, nullptr);
+    if (s != GLBE_OK) return s;
     GLBE2D_CUDA(cudaGetLastError(), "2D async error");
     return GLBE_OK;
 }

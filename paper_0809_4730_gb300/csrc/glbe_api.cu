@@ -283,7 +283,6 @@ namespace {
 // additions of a warp per row, then as many blocks as the grid needs (512 for
 // the 512 x 256 x 256 duct), and at most 16 more per row in the last block.
 constexpr int FIN_THREADS = 256;
-constexpr unsigned FIN_CHUNK = 256;
 
 __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(double* __restrict__ partials, unsigned nblocks,
                                                                const RecordOut out)
@@ -447,7 +446,8 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
     const long first = (c->t + 9) / 10 * 10;        // first residual level of the march
     m.have_snap = c->t_snap >= 0 && c->t_snap == first - 10;
     m.t0 = c->t;
-    m.nsteps = n;
+    m.phase = (int)(c->t % 10);
+    m.nsteps = (int)n;
     m.solve = solve ? 1 : 0;
     m.tol = tol;
     m.out = RecordOut{c->record, c->hist, c->hist_count, HIST_CAP, c->t_dev, c->stop_dev, c->tol_dev, c->mass0};
@@ -730,7 +730,13 @@ glbe_status glbe_step_n(glbe_ctx* c, long n)
     NvtxRange range_("glbe_step_n");
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(GLBE_ERR_ARG, "n must be >= 0");
-    if (c->res.form && n >= 2) return enqueue_resident(c, n, false, 0.0);
+    if (c->res.form && n >= 2) {
+        for (long k = 0; k < n; k += RES_MOST_STEPS) {
+            const glbe_status s = enqueue_resident(c, n - k < RES_MOST_STEPS ? n - k : RES_MOST_STEPS, false, 0.0);
+            if (s != GLBE_OK) return s;
+        }
+        return GLBE_OK;
+    }
     for (long k = 0; k < n; ++k) {
         glbe_status s = enqueue_step(c, c->stream, nullptr);
         if (s != GLBE_OK) return s;

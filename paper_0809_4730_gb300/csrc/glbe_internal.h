@@ -192,12 +192,16 @@ struct ResidentMarch {
     double* partials;
     int snap_lo;
     int have_snap;        // the snapshot is of the residual level before the first one of this march
-    long long t0, nsteps;
+    long long t0;
+    int phase;            // t0 mod 10
+    int nsteps;
     int solve;
     double tol;
     RecordOut out;
     unsigned* bar;        // barrier count, barrier generation, error flag
 };
+
+constexpr long RES_MOST_STEPS = 1000000;   // steps of one launch
 
 // How a grid's resident march is launched; form 0: it is not.
 struct ResidentPlan {

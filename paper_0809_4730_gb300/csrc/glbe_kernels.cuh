@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include "glbe_internal.h"
+#include "glbe_residual.cuh"
 
 namespace glbe {
 
@@ -1234,14 +1235,6 @@ __device__ __forceinline__ void node_update(const StepParams& p, const V (&d)[19
         if constexpr (COLL == 0) flow_collide<V, PRECISE>(p, mm, om, rho_inv, ns.jx, ns.jy, ns.jz, Fx, Fy, Fz);
         else srt_collide<V, PRECISE, COLL>(p, d, dl, S::COMP, om, ns.rho, ns.drho, ns.ux, ns.uy, ns.uz, Fx, Fy, Fz);
     }
-}
-
-template <typename V>
-__device__ __forceinline__ V warp_sum(V v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
 }
 
 // Residual sums of a block into partials[k][block]: FP32 per node, warp and

@@ -1,87 +1,30 @@
-// glbe_resident.cuh -- many time steps of a small grid in one launch.
+// glbe_resident.cuh -- many time steps of a small 3D grid in one launch
+// (glbe_resident_common.cuh): the gather tables, node updates and launch forms.
 //
 // A grid of at most a few nodes per resident thread is not bound by memory: a
 // launched step takes 8.5 us on every grid of up to 48^3 nodes (F32, flow),
 // most of it the launch itself, kernel prologue, geometry and the latency of
 // one gather.  Resident, a step takes (us, launched before -> resident):
 //                 F32 flow      F32 coupled   F32C flow     F32C coupled
-//   4 x 32 x 4    8.5 -> 2.2    8.5 -> 2.5    8.5 -> 2.4    10.0 -> 4.0
-//   64 x 64 x 8   8.7 -> 3.9    8.7 -> 4.4    8.5 -> 4.1    10.5 -> 5.7
-//   40^3          8.8 -> 4.6   10.8 -> 6.7   10.6 -> 5.9    14.6 -> 9.0
-//   64^3         14.4 -> 9.5   24.4 -> 17.9  20.6 -> 15.4   41.0 -> 30.6
-// Past about 70^3 the tables no longer leave the SM its full number of blocks
-// (72^3 coupled, F32, with a block less: 34.0 us, launched 32.6), and single
-// launches go on.  Here the blocks stay on their SMs
-// and march: each keeps a table of its nodes' gather slots in shared memory
-// (filled once: no geometry, no wall choice and no divergence in the loop),
-// updates its tiles from one population buffer into the other, and meets the
-// others at a barrier.  The node update is the step kernels' (node_from_sources),
-// so the states are theirs bit for bit.
-//
-// Two forms of the barrier:
-//   - CLUSTER (up to 16 blocks): the grid is one thread-block cluster and the
-//     hardware's cluster barrier orders the levels; the blocks are spread so
-//     that even the smallest grids use 16 SMs.  Residual sums travel through
-//     distributed shared memory.
-//   - otherwise a cooperative launch (all blocks resident) and a counting
-//     barrier in the workspace.  Every wait is bounded: a block that gives up
-//     raises an error flag, every block returns, and the host reports
-//     GLBE_ERR_TIMEOUT at its next synchronising call.
-//
-// Populations written earlier in the launch are gathered with ld.global.ca
-// (see ldp): the barrier's release and acquire order them.
+//   4 x 32 x 4    8.5 -> 2.2    8.5 -> 2.6    8.5 -> 2.3    10.0 -> 3.5
+//   64 x 64 x 8   8.7 -> 3.9    8.7 -> 4.6    8.5 -> 4.0    10.5 -> 5.7
+//   40^3          8.8 -> 4.4   10.8 -> 6.4   10.6 -> 5.6    14.6 -> 9.0
+//   64^3         13.2 -> 9.5   21.5 -> 17.5  17.7 -> 15.4   37.9 -> 31
+// (launched: with the reduction of glbe_residual.cuh).  The line lies where
+// the tables crowd out the gathers' L1 (RES_TABLES_FLOW, RES_TABLES_MHD):
+// 72^3 coupled marched 32.7 us a step with 205 KB of tables on an SM, 29.5
+// launched (F32C 56.3 and 52.7).  The node update is the step kernels'
+// (node_from_sources, pair_from_sources), so the states are theirs bit for bit.
 #pragma once
-#include <cooperative_groups.h>
-
-#include "glbe_residual.cuh"
+#include "glbe_resident_common.cuh"
 
 namespace glbe {
 
-constexpr int RES_THREADS = 256;        // nodes per tile, at most
 constexpr int RES_ROWS = 20;            // table rows: 19 slots and a flag word
-constexpr int RES_MAX_TILES = 8;        // tiles of a block, at most (its tables: 160 KB)
-constexpr size_t RES_TILE_BYTES = (size_t)RES_ROWS * RES_THREADS * sizeof(uint32_t);
-constexpr unsigned RES_SKIP = 0xffffffffu;   // flag word of a node that is not updated
-constexpr int RES_CLUSTER = 16;         // blocks of the cluster form
-constexpr unsigned RES_SPIN_LIMIT = 1u << 24;   // polls of a barrier wait, several seconds
-
-// Bounded counting barrier over the grid; gen is the caller's copy of the
-// barrier's generation (thread 0).  False once any block gave up.
-__device__ __forceinline__ bool resident_barrier(unsigned* bar, unsigned& gen)
-{
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned arrived;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(bar) : "memory");
-        int good = 1;
-        if (arrived == gridDim.x - 1) {
-            asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(bar + 1), "r"(gen + 1u) : "memory");
-        } else {
-            unsigned v, spins = 0;
-            while (true) {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar + 1) : "memory");
-                if (v != gen) break;
-                if (++spins > RES_SPIN_LIMIT || ((spins & 4095u) == 0 && *(volatile unsigned*)(bar + 2))) {
-                    atomicExch(bar + 2, 1u);
-                    good = 0;
-                    break;
-                }
-            }
-        }
-        ++gen;
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
-__device__ __forceinline__ void cluster_level_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+// Table bytes of an SM, at most: 9 tiles (64^3 F32C flow: 15.4 us a step with
+// them, 17.7 launched), 8 where a coupled node gathers f twice (64^3 F32C: 31
+// and 37.9 us; with 10 tiles the launched step is faster).
+constexpr size_t RES_TABLES_FLOW = (size_t)9 * RES_ROWS * 256 * 4, RES_TABLES_MHD = (size_t)8 * RES_ROWS * 256 * 4;
 
 // Slots of node i's gather in column tid of the table: row a holds the index
 // of direction a's source in a population buffer (its own opposite slot where
@@ -300,10 +243,9 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
     b.usnap = m.usnap;
     b.snap_lo = m.snap_lo;
     bool snap = m.have_snap != 0;               // the snapshot is of the previous residual level
-    for (long long s = 0; s < m.nsteps; ++s) {
-        const long long t = m.t0 + s;
-        const int par = (int)(t & 1);
-        const bool resid = t % 10 == 0;
+    int par = m.phase & 1;                      // t0 and t0 mod 10 have the same parity
+    for (int s = 0, phase = m.phase; s < m.nsteps; ++s, par ^= 1, phase = phase == 9 ? 0 : phase + 1) {
+        const bool resid = phase == 0;
         b.fsrc = m.f[par];
         b.fdst = m.f[par ^ 1];
         b.gsrc = m.g[par];
@@ -355,150 +297,57 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
                 // a solve's blocks all take the decision, from the same sums in the same order
                 for (int k = warp; k < RES_SUMS; k += BT / 32) {
                     if (!(writer || k < 2 || k == 6)) continue;
-                    const double v = CLUSTER ? partial_row_sum_shared(part + k * RES_CLUSTER, G)
+                    const double v = CLUSTER ? warp_sum_all(lane < G ? part[k * RES_CLUSTER + lane] : 0.0)
                                              : partial_row_sum(m.partials + (size_t)k * G, 0, (unsigned)G);
                     if (lane == 0) tot[k] = v;
                 }
                 __syncthreads();
                 if (threadIdx.x == 0) {
                     verdict = 0;
-                    if (m.solve) {
-                        const double r = residual_of(tot[0], tot[1]);
-                        verdict = (m.tol > 0.0 && r <= m.tol) || tot[6] > 0.0 || !isfinite(r);
-                    }
+                    if (m.solve) verdict = resident_stops(m.tol, tot);
                     if (writer && !*m.out.stop) write_record(m.out, tot, *m.out.t_dev);
                 }
                 __syncthreads();
                 if (verdict) return;            // the state is the one after level t, in every block
             } else if (!snap && writer && threadIdx.x == 0) {
-                *m.out.t_dev = t + 10;
+                *m.out.t_dev = m.t0 + s + 10;
             }
             snap = true;
         }
     }
 }
 
-// Blocks per SM at `per` tiles a block, asked of the runtime once per kernel.
-template <int ST, bool MHD, bool PAIR, bool DENSE>
-int resident_blocks_per_sm(int per)
-{
-    static const auto occ = [] {
-        struct { int n[RES_MAX_TILES + 1]; } r{};
-        auto* kernel = resident_kernel<ST, MHD, PAIR, DENSE, false>;
-        for (int k = 1; k <= RES_MAX_TILES; ++k)
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.n[k], kernel, RES_THREADS, k * RES_TILE_BYTES) !=
-                cudaSuccess)
-                r.n[k] = 0;
-        cudaGetLastError();
-        return r;
-    }();
-    return per <= RES_MAX_TILES ? occ.n[per] : 0;
-}
-
-template <int ST, bool MHD, bool PAIR>
-bool resident_cluster_fits()
-{
-    static const bool fits = [] {
-        auto* kernel = resident_kernel<ST, MHD, PAIR, false, true>;
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = RES_CLUSTER;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(RES_CLUSTER);
-        cfg.blockDim = dim3(RES_THREADS);
-        cfg.dynamicSmemBytes = RES_TILE_BYTES;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        const bool ok = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
-        cudaGetLastError();
-        return ok;
-    }();
-    return fits;
-}
-
-template <int ST, bool MHD, bool PAIR, bool DENSE>
-bool resident_grid_plan(uint32_t N, int sms, int max_per, ResidentPlan* out)
-{
-    // the fewest tiles per block at which all blocks are resident, while the
-    // tables leave the SM its full number of blocks
-    const int full = resident_blocks_per_sm<ST, MHD, PAIR, DENSE>(1);
-    for (int per = 1; per <= max_per && resident_blocks_per_sm<ST, MHD, PAIR, DENSE>(per) == full; ++per) {
-        const long long room = (long long)full * sms;
-        const uint32_t tiles = ((PAIR && DENSE ? N >> 1 : N) + RES_THREADS - 1) / RES_THREADS;
-        if (room * per < tiles) continue;
-        *out = {DENSE ? 3 : 2, PAIR ? 1 : 0, (int)(room < tiles ? room : tiles), RES_THREADS,
-                (unsigned)(per * RES_TILE_BYTES)};
-        return true;
-    }
-    return false;
-}
-
 template <int ST, bool MHD, bool PAIR>
 cudaError_t resident_plan_t(uint32_t N, ResidentPlan* out)
 {
-    int dev = 0, sms = 0, coop = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    if ((long long)N > (long long)RES_MAX_TILES * sms * 4 * RES_THREADS) return cudaSuccess;   // more tables than shared memory
-    // the limits are function attributes of the device: the same values whoever sets them
-    const int most = RES_MAX_TILES * (int)RES_TILE_BYTES;
-    e = cudaFuncSetAttribute(resident_kernel<ST, MHD, PAIR, false, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(resident_kernel<ST, MHD, PAIR, false, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(resident_kernel<ST, MHD, PAIR, true, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e != cudaSuccess) return e;
-    if (N <= (uint32_t)RES_CLUSTER * RES_THREADS && resident_cluster_fits<ST, MHD, PAIR>()) {
-        const int threads = 32 * (int)((N + RES_CLUSTER * 32 - 1) / (RES_CLUSTER * 32));
-        *out = {1, PAIR ? 1 : 0, RES_CLUSTER, threads, (unsigned)(RES_ROWS * threads * sizeof(uint32_t))};
-        return cudaSuccess;
-    }
-    if (!coop) return cudaSuccess;
-    if (resident_grid_plan<ST, MHD, PAIR, false>(N, sms, 1, out)) return cudaSuccess;
-    resident_grid_plan<ST, MHD, PAIR, true>(N, sms, RES_MAX_TILES, out);
-    return cudaSuccess;
-}
-
-template <int ST, bool MHD, bool PAIR, bool DENSE, bool CLUSTER>
-cudaError_t resident_launch(const StepParams& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
-{
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    if (CLUSTER) {
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = RES_CLUSTER;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    } else {
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-    }
-    cfg.gridDim = dim3(pl.blocks);
-    cfg.blockDim = dim3(pl.threads);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, resident_kernel<ST, MHD, PAIR, DENSE, CLUSTER>, p, m);
+    constexpr size_t tile = (size_t)RES_ROWS * RES_THREADS * sizeof(uint32_t);
+    auto* cluster = resident_kernel<ST, MHD, PAIR, false, true>;
+    auto* free_form = resident_kernel<ST, MHD, PAIR, false, false>;
+    auto* dense = resident_kernel<ST, MHD, PAIR, true, false>;
+    static const ResidentOcc of = resident_occupancy(free_form, tile), od = resident_occupancy(dense, tile);
+    static const bool fits = [&] {
+        cudaFuncSetAttribute(cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return resident_cluster_fits(cluster, tile);
+    }();
+    const cudaError_t e = resident_plan_of(cluster, free_form, dense, N, PAIR ? N >> 1 : N, RES_ROWS,
+                                           MHD ? RES_TABLES_MHD : RES_TABLES_FLOW, of, od, fits, out);
+    out->pair = PAIR ? 1 : 0;
+    return e;
 }
 
 template <int ST, bool MHD, bool PAIR>
 cudaError_t resident_march_t(const StepParams& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
 {
-    if (pl.form == 1) return resident_launch<ST, MHD, PAIR, false, true>(p, m, pl, st);
-    if (pl.form == 2) return resident_launch<ST, MHD, PAIR, false, false>(p, m, pl, st);
-    return resident_launch<ST, MHD, PAIR, true, false>(p, m, pl, st);
+    if (pl.form == 1) return resident_launch(resident_kernel<ST, MHD, PAIR, false, true>, pl, st, p, m);
+    if (pl.form == 2) return resident_launch(resident_kernel<ST, MHD, PAIR, false, false>, pl, st, p, m);
+    return resident_launch(resident_kernel<ST, MHD, PAIR, true, false>, pl, st, p, m);
 }
 
 template <int ST>
 cudaError_t resident_plan(bool mhd, const StepParams& p, ResidentPlan* out)
 {
     *out = ResidentPlan{0, 0, 0, 0, 0};
+    if (p.N > RES_MAX_NODES) return cudaSuccess;
     if (mhd) return resident_plan_t<ST, true, false>(p.N, out);
     if constexpr (!Store<ST>::COMP) {
         if (pair_eligible(p, mhd, MODE_STEP)) return resident_plan_t<ST, false, true>(p.N, out);

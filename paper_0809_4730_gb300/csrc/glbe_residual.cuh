@@ -16,7 +16,24 @@
 
 namespace glbe {
 
+template <typename V>
+__device__ __forceinline__ V warp_sum(V v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+
 constexpr int RES_SUMS = 7;   // num, den, sum drho, Mx, My, Mz, non-finite count
+
+constexpr unsigned FIN_CHUNK = 256;   // partials that one block (or pass) sums
+
+__device__ __forceinline__ double warp_sum_all(double t)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
 
 // Sum of row[b0, b1) by one warp, in every lane: a fixed order.  Reads through
 // L2 (the partials may have been written earlier in the same launch).
@@ -25,6 +42,7 @@ __device__ __forceinline__ double partial_row_sum(const double* row, unsigned b0
     const unsigned lane = threadIdx.x & 31u;
     double s[4] = {0.0, 0.0, 0.0, 0.0};
     unsigned b = b0 + lane;
+#pragma unroll 2
     for (; b + 96u < b1; b += 128u) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) s[k] += __ldcg(row + b + 32u * k);
@@ -32,20 +50,7 @@ __device__ __forceinline__ double partial_row_sum(const double* row, unsigned b0
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         if (b + 32u * k < b1) s[k] += __ldcg(row + b + 32u * k);
-    double t = (s[0] + s[1]) + (s[2] + s[3]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    return t;
-}
-
-// The same of at most 32 values in shared memory.
-__device__ __forceinline__ double partial_row_sum_shared(const double* row, int n)
-{
-    const int lane = threadIdx.x & 31;
-    double t = lane < n ? row[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    return t;
+    return warp_sum_all((s[0] + s[1]) + (s[2] + s[3]));
 }
 
 // r(t) of the sums (Sec. 5): ||u(t) - u(t-10)|| / ||u(t)||.

@@ -111,6 +111,50 @@ def test_divergence_ends_a_solve_and_is_reported(shape):
     S.close()
 
 
+# 2D: one cluster and past it, one tile on each of 152 SMs and past it, several tiles a block, the largest of
+# the dense forms and past them
+SHAPES2 = [((1, 5), "y"), ((64, 64), "y"), ((65, 64), "xy"), ((128, 304), "y"), ((129, 304), ""), ((333, 501), "x"),
+           ((700, 700), "y"), ((1100, 1000), "y")]
+
+
+@pytest.mark.parametrize("mhd", [False, True])
+@pytest.mark.parametrize("storage", ["f32", "f32c", "bf16"])
+def test_2d_march_equals_single_steps(storage, mhd):
+    import torch
+    from paper_0809_4730_gb300.glbe import Solver2D
+    for shape, walls in SHAPES2:
+        w = tuple(int(c in walls) for c in "xy")
+        kw = dict(wall_lo=w, wall_hi=w, gamma=0.2, nu=0.05, F=(2e-6, 1e-6), storage=storage)
+        if mhd:
+            kw.update(induction=1, gamma_m=0.2, eta=0.05, chi=0.05, mu=1.0, B0=(0.002, 0.004))
+        A, B = Solver2D(*shape, **kw), Solver2D(*shape, **kw)
+        g = torch.Generator(device="cuda").manual_seed(3)
+        r = lambda q, s: s * (2 * torch.rand(q, A.N, device="cuda", generator=g) - 1)  # noqa: E731
+        st = (r(9, 1e-4), r(10, 1e-5) if mhd else None, r(2, 1e-7) if mhd else None, 0)
+        A.set_state(*st)
+        B.set_state(*st)
+        A.step(2)
+        A.step(21)
+        for _ in range(23):
+            B.step(1)
+        _same(A.get_state(), B.get_state())
+        # the same FP32 partials; their FP64 sum in another order past one cluster
+        ha, hb = A.history(), B.history()
+        assert [h.t for h in ha] == [h.t for h in hb] == [10, 20]
+        for x, y in zip(ha, hb):
+            rel = 0.0 if A.N <= 4096 else 1e-13
+            assert abs(x.num - y.num) <= rel * y.num and abs(x.den - y.den) <= rel * y.den
+            assert abs(x.r - y.r) <= rel * y.r and abs(x.mass - y.mass) <= rel * y.mass
+        # a capped solve takes every step
+        status, t, _ = A.solve(1e-30, 18)
+        assert status == 4 and t == 41
+        for _ in range(18):
+            B.step(1)
+        _same(A.get_state(), B.get_state())
+        A.close()
+        B.close()
+
+
 def test_two_streams_march_apart():
     import torch
     out = []
