@@ -171,9 +171,8 @@ __global__ void __launch_bounds__(BT, 512 / BT) batch_kernel(const BatchDomain* 
                 // within the kernel's register budget; the one-pass update
                 // spilled over a kilobyte per thread.
                 if (mhd) {
-                    coupled_induction_pass<ST, true>(sp, b, i);
-                    if (resid) scalar_node_step<ST, false, MODE_STEP_RESID, true, false, true>(sp, b, fo, i, acc);
-                    else scalar_node_step<ST, false, MODE_STEP, true, false, true>(sp, b, fo, i, acc);
+                    if (resid) coupled_node2<ST, MODE_STEP_RESID, true>(sp, b, i, acc);
+                    else coupled_node2<ST, MODE_STEP, true>(sp, b, i, acc);
                 } else {
                     if (resid) scalar_node_step<ST, false, MODE_STEP_RESID, true>(sp, b, fo, i, acc);
                     else scalar_node_step<ST, false, MODE_STEP, true>(sp, b, fo, i, acc);

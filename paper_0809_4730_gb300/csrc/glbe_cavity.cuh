@@ -30,7 +30,9 @@ __device__ __forceinline__ bool in_box(const StepParams& p, int x, int y, int z)
 // induction part and the flow part are each in the kernel once.  (A form with
 // separate gathers for nodes inside the box and one induction part for each
 // side of its boundary was bound by instruction fetch: 2.6 stalled cycles per
-// issued instruction; the F32C step of the 98^3 MHD cavity took 152 us.)
+// issued instruction; the F32C step of the 98^3 MHD cavity took 152 us.  Now 98
+// us: bound by the latency of its gathers, hence 24 warps an SM in spite of
+// 216 B spilled (two blocks, no spill: 109 us) and the L2 prefetch.)
 struct CavGeo {
     uint32_t n;
     uint32_t off[3][3];
@@ -193,6 +195,21 @@ __global__ void __launch_bounds__(STEP_THREADS) cavity_kernel(const StepParams p
     if (MODE == MODE_STEP_RESID) block_partials<STEP_THREADS>(acc, b.partials);
 }
 
+// Whether the block that this one prefetches for may hold nodes of the flow
+// lattice: its rows meet the box's in z and, when it lies within one z plane,
+// in y.
+__device__ __forceinline__ bool box_ahead(const StepParams& p, const StepBuffers& b)
+{
+    const long long first = ((long long)blockIdx.x + b.pf_ahead) * STEP_THREADS;
+    if (first >= (long long)p.N) return false;
+    const uint32_t n0 = (uint32_t)first, n1 = n0 + STEP_THREADS - 1 < p.N ? n0 + STEP_THREADS - 1 : p.N - 1;
+    const int z0 = (int)fdiv(n0, p.div_nxy), z1 = (int)fdiv(n1, p.div_nxy);
+    if (z1 < p.blo[2] || z0 > p.bhi[2]) return false;
+    if (z0 != z1) return true;
+    const int y0 = (int)fdiv(n0, p.div_nx) - z0 * p.ny, y1 = (int)fdiv(n1, p.div_nx) - z1 * p.ny;
+    return y1 >= p.blo[1] && y0 <= p.bhi[1];
+}
+
 // The coupled cavity step in two passes per thread (the FP32 forms; the
 // one-pass coupled F32C update needs 172 registers, one block per SM): pass 1
 // gathers g, and f at a node of the flow lattice, for rho and m (at rest
@@ -201,27 +218,29 @@ __global__ void __launch_bounds__(STEP_THREADS) cavity_kernel(const StepParams p
 // update with F = F_ext + F_L.  The one-pass arithmetic in the same order, bit
 // for bit.
 template <int ST, int MODE>
-__global__ void __launch_bounds__(STEP_THREADS, 2) cavity_kernel_coupled2(const StepParams p, const StepBuffers b,
+__global__ void __launch_bounds__(STEP_THREADS, 3) cavity_kernel_coupled2(const StepParams p, const StepBuffers b,
                                                                            const FieldOut fo)
 {
     using T = typename Store<ST>::T;
     constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
     if (b.stop != nullptr && *b.stop) return;
+    prefetch_ahead<ST, STEP_THREADS, true, MODE == MODE_STEP_RESID>(p, b, box_ahead(p, b));
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i < p.N) {
         const CavGeo g = cavity_geo(p, i);
         if (!g.solid) {
-            float q[21], ql[21], og[21];
-            load_g_box<ST>(p, static_cast<const T*>(b.gsrc), g, q, ql);
             float rho_inv = 1.f, mx = 0.f, my = 0.f, mz = 0.f;
             NodeIn<float> in{};
             if (g.flow) {
                 float d[19], dl[19];
-                load_f_box<ST>(p, static_cast<const T*>(b.fsrc), g, d, dl);
                 in = node_inputs<true, MODE_STEP>(p, b, i);
+                load_f_box<ST>(p, static_cast<const T*>(b.fsrc), g, d, dl);
                 node_momentum<ST>(p, d, dl, rho_inv, mx, my, mz);
             }
+            f_before_g();
+            float q[21], ql[21], og[21];
+            load_g_box<ST>(p, static_cast<const T*>(b.gsrc), g, q, ql);
             NodeMacro<float> mac;
             induction_collide<float, PRECISE, Store<ST>::COMP>(p, q, ql, og, rho_inv, mx, my, mz, in.Fx, in.Fy, in.Fz,
                                                               in.FLx, in.FLy, in.FLz, mac);

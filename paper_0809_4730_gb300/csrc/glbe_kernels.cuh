@@ -773,6 +773,61 @@ __device__ __forceinline__ void split_exact(const V& x, V& xh, V& xl)
     xl = vsub_rn(x, xh);
 }
 
+// The exact split of Q values, each low part plus (COMP) the compensated
+// storage's.  One node's values go two at a time through the packed operations:
+// these are additions and subtractions only, each lane rounded as a scalar one
+// is, so the bits are the scalar split's at half the instructions (with
+// store_comp_rows 1130 -> 998 instructions a node of the F32C flow step and
+// 0.0873 -> 0.0834 ms on a 128^3 duct).  (Not PACK:
+// one by one, for the resident marches, where a level is a chain of latencies
+// and the packed operations lengthen it: 64 x 64 x 8 F32C coupled 5.6 against
+// 5.9 us a step.)
+template <bool COMP, bool PACK, int Q>
+__device__ __forceinline__ void split_rows(const float (&x)[Q], const float (&xlo)[Q], float (&h)[Q], float (&l)[Q])
+{
+    if constexpr (!PACK) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            split_exact(x[i], h[i], l[i]);
+            if constexpr (COMP) l[i] += xlo[i];
+        }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i + 1 < Q; i += 2) {
+        const F2 v(x[i], x[i + 1]);
+        F2 vh, vl;
+        split_exact(v, vh, vl);
+        if constexpr (COMP) vl += F2(xlo[i], xlo[i + 1]);
+        h[i] = vh.v.x;
+        h[i + 1] = vh.v.y;
+        l[i] = vl.v.x;
+        l[i + 1] = vl.v.y;
+    }
+    if constexpr (Q % 2 == 1) {
+        split_exact(x[Q - 1], h[Q - 1], l[Q - 1]);
+        if constexpr (COMP) l[Q - 1] += xlo[Q - 1];
+    }
+}
+template <bool COMP, bool, int Q>
+__device__ __forceinline__ void split_rows(const F2 (&x)[Q], const F2 (&xlo)[Q], F2 (&h)[Q], F2 (&l)[Q])
+{
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        split_exact(x[i], h[i], l[i]);
+        if constexpr (COMP) l[i] += xlo[i];
+    }
+}
+template <bool COMP, bool, int Q>
+__device__ __forceinline__ void split_rows(const F1 (&x)[Q], const F1 (&xlo)[Q], F1 (&h)[Q], F1 (&l)[Q])
+{
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        split_exact(x[i], h[i], l[i]);
+        if constexpr (COMP) l[i] += xlo[i];
+    }
+}
+
 // Everything the induction part produces besides the new populations.
 template <class V>
 struct NodeMacro {
@@ -788,19 +843,13 @@ struct NodeMacro {
 // first bracket is exact and the rounding of the 7-term sum B no longer
 // biases every population's relaxation (a bias the slow magnetic diffusion
 // mode would otherwise integrate into a 3e-5 error of the steady flow).
-template <class V, bool PRECISE, bool COMP>
+template <class V, bool PRECISE, bool COMP, bool PACK = true>
 __device__ __forceinline__ void induction_collide(const StepParams& p, const V (&q)[21], const V (&qlo)[21],
                                                   V (&og)[21], V rho_inv, V mx, V my, V mz, V Fx, V Fy, V Fz,
                                                   V FLpx, V FLpy, V FLpz, NodeMacro<V>& mac)
 {
     V qh[21], ql[21];
-    if constexpr (PRECISE) {
-#pragma unroll
-        for (int i = 0; i < 21; ++i) {
-            split_exact(q[i], qh[i], ql[i]);
-            if constexpr (COMP) ql[i] += qlo[i];   // low part of the compensated storage
-        }
-    }
+    if constexpr (PRECISE) split_rows<COMP, PACK>(q, qlo, qh, ql);
     // B_j = B0_j + sum_a dg_ja (sum_a W_a = 1), Eq. magneticinduction
     V bxh, byh, bzh, bxl(0.f), byl(0.f), bzl(0.f);
     if constexpr (PRECISE) {
@@ -1168,7 +1217,7 @@ struct NodeState {
 // The whole update of a node (pair) from its gathered populations: moments,
 // induction and Lorentz force, velocity, collision changes om (f) and og (g).
 // With collide = false only the macroscopic fields are formed.
-template <class V, int ST, bool MHD, int COLL = 0>
+template <class V, int ST, bool MHD, int COLL = 0, bool PACK = true>
 __device__ __forceinline__ void node_update(const StepParams& p, const V (&d)[19], const V (&dl)[19],
                                             const V (&q)[21], const V (&ql)[21], V FLpx, V FLpy, V FLpz, V Fx,
                                             V Fy, V Fz, bool collide, V (&om)[19], V (&og)[21], NodeState<V>& ns)
@@ -1180,11 +1229,7 @@ __device__ __forceinline__ void node_update(const StepParams& p, const V (&d)[19
     NodeMoments<V, PRECISE> mm;
     if constexpr (PRECISE) {
         V dh[19], dlo[19];
-#pragma unroll
-        for (int a = 0; a < 19; ++a) {
-            split_exact(d[a], dh[a], dlo[a]);
-            if constexpr (S::COMP) dlo[a] += dl[a];
-        }
+        split_rows<S::COMP, PACK>(d, dl, dh, dlo);
         mm.H = linear_moments(dh);
         mm.L = linear_moments(dlo);
     } else {
@@ -1198,7 +1243,7 @@ __device__ __forceinline__ void node_update(const StepParams& p, const V (&d)[19
     ns.mac.Bx = ns.mac.By = ns.mac.Bz = V(0.f);
     ns.mac.FLx = ns.mac.FLy = ns.mac.FLz = V(0.f);
     if (MHD) {
-        induction_collide<V, PRECISE, S::COMP>(p, q, ql, og, rho_inv, PRECISE ? mxh + mxl : mxh,
+        induction_collide<V, PRECISE, S::COMP, PACK>(p, q, ql, og, rho_inv, PRECISE ? mxh + mxl : mxh,
                                                PRECISE ? myh + myl : myh, PRECISE ? mzh + mzl : mzh, Fx, Fy, Fz,
                                                FLpx, FLpy, FLpz, ns.mac);
         Fx += ns.mac.FLx;
@@ -1354,7 +1399,7 @@ __device__ __forceinline__ NodeIn<V> pair_inputs(const StepParams& p, const Step
     return in;
 }
 
-template <int ST, bool MHD, int MODE, bool DIR = false, int COLL = 0>
+template <int ST, bool MHD, int MODE, bool DIR = false, int COLL = 0, bool PACK = true>
 __device__ __forceinline__ void node_from_sources(const StepParams& p, const StepBuffers& b, const FieldOut& fo,
                                                   uint32_t n, const float (&d)[19], const float (&dl)[19],
                                                   const float (&q)[21], const float (&ql)[21],
@@ -1381,7 +1426,7 @@ __device__ __forceinline__ void load_f_interior_dir(const StepParams& p, const S
 // of MODE_STEP_RESID into acc.  Returns without work for solid nodes.
 // DIR: the per-direction bases of b are filled (kernels launched by
 // launch_mode); they serve the interior gather and the stores of f.
-template <int ST, bool MHD, int MODE, bool CG = false, bool DIR = false, bool FL_IN_F = false, int COLL = 0>
+template <int ST, bool MHD, int MODE, bool CG = false, bool DIR = false, int COLL = 0>
 __device__ __forceinline__ void scalar_node_step(const StepParams& p, const StepBuffers& b, const FieldOut& fo,
                                                  uint32_t i, float (&acc)[7])
 {
@@ -1411,49 +1456,65 @@ __device__ __forceinline__ void scalar_node_step(const StepParams& p, const Step
         load_f<ST, CG>(p, static_cast<const T*>(b.fsrc), g, d, dl);
         if (MHD) load_g<ST, CG>(p, static_cast<const T*>(b.gsrc), g, q, ql);
     }
-    node_from_sources<ST, MHD, MODE, DIR, COLL>(p, b, fo, n, d, dl, q, ql, node_inputs<MHD, MODE, FL_IN_F>(p, b, n),
-                                                 acc);
+    node_from_sources<ST, MHD, MODE, DIR, COLL>(p, b, fo, n, d, dl, q, ql, node_inputs<MHD, MODE>(p, b, n), acc);
 }
 
-// Two-pass coupled update, pass 1 (the persistent batch kernel: one update
-// of a coupled node does not fit its register budget).  Gathers f and g of
-// node i, forms rho and m (Eq. precondhydrofields), runs the induction part
-// exactly as node_update does (B, Lorentz force from the previous step's
-// half-force velocity, D3Q7 collision; Sec. 4) and writes g~ and this step's
-// Lorentz force into b.FL.  Pass 2 is scalar_node_step<ST, false, MODE, CG,
-// false, true>: it gathers f again (from L2) and runs the flow update with
-// F = F_ext + b.FL, which is the one-pass update's arithmetic in the same
-// order, so the result is bit for bit the same.
-template <int ST>
+// Two-pass coupled update (coupled_node2): pass 1 forms rho and m from f (Eq.
+// precondhydrofields), runs the induction part exactly as node_update does (B,
+// Lorentz force from the previous step's half-force velocity, D3Q7 collision;
+// Sec. 4) and writes g~ and this step's Lorentz force into b.FL; pass 2 runs
+// the flow update with F = F_ext + b.FL, which is the one-pass update's
+// arithmetic in the same order, so the result is bit for bit the same.
+template <int ST, bool PACK = true>
+__device__ __forceinline__ void node_momentum(const StepParams& p, const float (&d)[19], const float (&dl)[19],
+                                              float& rho_inv, float& mx, float& my, float& mz);
+template <int ST, bool PACK = true>
 __device__ __forceinline__ void induction_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n,
-                                                      const float (&d)[19], const float (&dl)[19],
-                                                      const float (&q)[21], const float (&ql)[21]);
+                                                      const NodeIn<float>& in, float rho_inv, float mx, float my,
+                                                      float mz, const float (&q)[21], const float (&ql)[21]);
+// f is down to rho and m before any of g is gathered: the empty asm keeps the
+// loads of g behind it, or the 80 values of both would be live together.
+__device__ __forceinline__ void f_before_g() { asm volatile("" ::: "memory"); }
 
-template <int ST, bool CG>
-__device__ __forceinline__ void coupled_induction_pass(const StepParams& p, const StepBuffers& b, uint32_t i)
+// The compensated sums old + change of Q populations of node n into rows of N
+// high parts (hi) and, behind them, of N low parts: additions and subtractions
+// only, so two rows at a time in the packed operations (see split_rows).
+template <bool PACK, int Q>
+__device__ __forceinline__ void store_comp_rows(float* hi, size_t N, uint32_t n, const float (&v)[Q],
+                                                const float (&vl)[Q], const float (&o)[Q])
 {
-    using S = Store<ST>;
-    using T = typename S::T;
-    constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
-    if (!(i < p.N)) return;
-    const uint32_t n = i;
-    const size_t N = p.N;
-    float d[19], dl[19], q[21], ql[21];
-    int wp = 0, wm = 0;
-    if (is_interior(p, n, wp, wm)) {
-        load_f_interior<ST, CG>(p, static_cast<const T*>(b.fsrc), n, wp, wm, d, dl);
-        load_g_interior<ST, CG>(p, static_cast<const T*>(b.gsrc), n, wp, wm, q, ql);
-    } else {
-        const Geo g = make_geo(p, n);
-        if (g.solid) return;
-        load_f<ST, CG>(p, static_cast<const T*>(b.fsrc), g, d, dl);
-        load_g<ST, CG>(p, static_cast<const T*>(b.gsrc), g, q, ql);
+    __half* lo = reinterpret_cast<__half*>(hi + Q * N);
+    if constexpr (!PACK) {
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            float nh, nl;
+            comp_add(v[a], vl[a], o[a], nh, nl);
+            hi[(size_t)a * N + n] = nh;
+            lo[(size_t)a * N + n] = Store<ST_F32C>::cv_lo(nl);
+        }
+        return;
     }
-    induction_from_sources<ST>(p, b, n, d, dl, q, ql);
+#pragma unroll
+    for (int a = 0; a + 1 < Q; a += 2) {
+        F2 nh, nl;
+        comp_add(F2(v[a], v[a + 1]), F2(vl[a], vl[a + 1]), F2(o[a], o[a + 1]), nh, nl);
+        nl = nl * F2(LO_SCALE);
+        hi[(size_t)a * N + n] = nh.v.x;
+        hi[(size_t)(a + 1) * N + n] = nh.v.y;
+        const __half2 w = __float22half2_rn(nl.v);
+        lo[(size_t)a * N + n] = __low2half(w);
+        lo[(size_t)(a + 1) * N + n] = __high2half(w);
+    }
+    if constexpr (Q % 2 == 1) {
+        float nh, nl;
+        comp_add(v[Q - 1], vl[Q - 1], o[Q - 1], nh, nl);
+        hi[(size_t)(Q - 1) * N + n] = nh;
+        lo[(size_t)(Q - 1) * N + n] = Store<ST_F32C>::cv_lo(nl);
+    }
 }
 
 // 1/rho and m of a node's gathered f, as node_update forms them.
-template <int ST>
+template <int ST, bool PACK>
 __device__ __forceinline__ void node_momentum(const StepParams& p, const float (&d)[19], const float (&dl)[19],
                                               float& rho_inv, float& mx, float& my, float& mz)
 {
@@ -1461,11 +1522,7 @@ __device__ __forceinline__ void node_momentum(const StepParams& p, const float (
     NodeMoments<float, PRECISE> mm;
     if constexpr (PRECISE) {
         float dh[19], dlo[19];
-#pragma unroll
-        for (int a = 0; a < 19; ++a) {
-            split_exact(d[a], dh[a], dlo[a]);
-            if constexpr (Store<ST>::COMP) dlo[a] += dl[a];
-        }
+        split_rows<Store<ST>::COMP, PACK>(d, dl, dh, dlo);
         mm.H = linear_moments(dh);
         mm.L = linear_moments(dlo);
     } else {
@@ -1479,7 +1536,7 @@ __device__ __forceinline__ void node_momentum(const StepParams& p, const float (
 }
 
 // g~ = g + og into node n's own slots, and this step's Lorentz force.
-template <int ST>
+template <int ST, bool PACK = true>
 __device__ __forceinline__ void store_induction(const StepParams& p, const StepBuffers& b, uint32_t n,
                                                 const float (&q)[21], const float (&ql)[21], const float (&og)[21],
                                                 float FLx, float FLy, float FLz)
@@ -1489,14 +1546,7 @@ __device__ __forceinline__ void store_induction(const StepParams& p, const StepB
     const size_t N = p.N;
     T* __restrict__ gd = static_cast<T*>(b.gdst);
     if constexpr (S::COMP) {
-        __half* __restrict__ gdl = reinterpret_cast<__half*>(gd + 21 * N);
-#pragma unroll
-        for (int a = 0; a < 21; ++a) {
-            float nh, nl;
-            comp_add(q[a], ql[a], og[a], nh, nl);
-            gd[(size_t)a * N + n] = nh;
-            gdl[(size_t)a * N + n] = S::cv_lo(nl);
-        }
+        store_comp_rows<PACK>(gd, N, n, q, ql, og);
     } else {
 #pragma unroll
         for (int a = 0; a < 21; ++a) gd[(size_t)a * N + n] = S::cv(toscale<ST>(p, q[a] + og[a]));
@@ -1506,23 +1556,19 @@ __device__ __forceinline__ void store_induction(const StepParams& p, const StepB
     b.FL[2 * N + n] = FLz;
 }
 
-// Pass 1 of the two-pass coupled update from the gathered populations of
-// node n: rho and m, the induction part, and the stores of g~ and of this
-// step's Lorentz force.
-template <int ST>
+// Pass 1 of the two-pass coupled update of node n from its inputs (loaded by the
+// caller, ahead of the gathers they are used after), rho, m and gathered g: the induction part, and the stores of g~ and of this step's Lorentz force.
+template <int ST, bool PACK>
 __device__ __forceinline__ void induction_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n,
-                                                      const float (&d)[19], const float (&dl)[19],
-                                                      const float (&q)[21], const float (&ql)[21])
+                                                      const NodeIn<float>& in, float rho_inv, float mx, float my,
+                                                      float mz, const float (&q)[21], const float (&ql)[21])
 {
     constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
-    const NodeIn<float> in = node_inputs<true, MODE_STEP>(p, b, n);
-    float rho_inv, mx, my, mz;
-    node_momentum<ST>(p, d, dl, rho_inv, mx, my, mz);
     float og[21];
     NodeMacro<float> mac;
-    induction_collide<float, PRECISE, Store<ST>::COMP>(p, q, ql, og, rho_inv, mx, my, mz, in.Fx, in.Fy, in.Fz, in.FLx,
-                                                      in.FLy, in.FLz, mac);
-    store_induction<ST>(p, b, n, q, ql, og, mac.FLx, mac.FLy, mac.FLz);
+    induction_collide<float, PRECISE, Store<ST>::COMP, PACK>(p, q, ql, og, rho_inv, mx, my, mz, in.Fx, in.Fy, in.Fz,
+                                                            in.FLx, in.FLy, in.FLz, mac);
+    store_induction<ST, PACK>(p, b, n, q, ql, og, mac.FLx, mac.FLy, mac.FLz);
 }
 
 // The update of fluid node n from its gathered pre-collision populations
@@ -1530,7 +1576,7 @@ __device__ __forceinline__ void induction_from_sources(const StepParams& p, cons
 // force and the force field, collides, writes the node's own slots of the
 // destination buffers (or the fields in MODE_FIELDS) and adds the residual
 // terms of MODE_STEP_RESID to acc.
-template <int ST, bool MHD, int MODE, bool DIR, int COLL>
+template <int ST, bool MHD, int MODE, bool DIR, int COLL, bool PACK>
 __device__ __forceinline__ void node_from_sources(const StepParams& p, const StepBuffers& b, const FieldOut& fo,
                                                   uint32_t n, const float (&d)[19], const float (&dl)[19],
                                                   const float (&q)[21], const float (&ql)[21],
@@ -1541,7 +1587,7 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
     const size_t N = p.N;
     float om[19], og[21];
     NodeState<float> ns;
-    node_update<float, ST, MHD, COLL>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz, MODE != MODE_FIELDS, om,
+    node_update<float, ST, MHD, COLL, PACK>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz, MODE != MODE_FIELDS, om,
                                 og, ns);
 
     if (MODE == MODE_FIELDS) {
@@ -1554,14 +1600,7 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
     T* __restrict__ fd = static_cast<T*>(b.fdst);
     [[maybe_unused]] SrBits rb(n, step_seed<ST>(b));
     if constexpr (S::COMP) {
-        __half* __restrict__ fdl = reinterpret_cast<__half*>(fd + 19 * N);
-#pragma unroll
-        for (int a = 0; a < 19; ++a) {
-            float nh, nl;
-            comp_add(d[a], dl[a], om[a], nh, nl);
-            fd[(size_t)a * N + n] = nh;
-            fdl[(size_t)a * N + n] = S::cv_lo(nl);
-        }
+        store_comp_rows<PACK>(fd, N, n, d, dl, om);
     } else if constexpr (DIR) {
 #pragma unroll
         for (int a = 0; a < 19; ++a)
@@ -1573,14 +1612,7 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
     if (MHD) {
         T* __restrict__ gd = static_cast<T*>(b.gdst);
         if constexpr (S::COMP) {
-            __half* __restrict__ gdl = reinterpret_cast<__half*>(gd + 21 * N);
-#pragma unroll
-            for (int a = 0; a < 21; ++a) {
-                float nh, nl;
-                comp_add(q[a], ql[a], og[a], nh, nl);
-                gd[(size_t)a * N + n] = nh;
-                gdl[(size_t)a * N + n] = S::cv_lo(nl);
-            }
+            store_comp_rows<PACK>(gd, N, n, q, ql, og);
         } else {
 #pragma unroll
             for (int a = 0; a < 21; ++a) gd[(size_t)a * N + n] = store_cv<ST>(toscale<ST>(p, q[a] + og[a]), rb);
@@ -1615,6 +1647,60 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
     }
 }
 
+// The two-pass coupled update of node i: f is gathered for rho and m, then g
+// for the induction part, then f again (from L1 / L2) for the flow update.
+// Interior and other nodes differ only in the gathers, so each part is in the
+// kernel once; the other nodes' geometry is formed anew for each gather (the
+// empty asm keeps the compiler from carrying it) rather than held in registers
+// across them.  With the parts in the kernel twice (an interior and a general
+// one each) it stalled on instruction fetch 1.2 cycles per issued instruction
+// and took 2473 of them a node, 2174 now; what bounds it now is the latency of
+// the three gathers at 16 warps an SM.  F32C, launched: 72^3 52.7 -> 48.7 us a
+// step, 96^3 105 -> 97 us; 64 batched ducts 9.05 -> 8.33 ms a level.  Held to
+// three blocks (80 registers) it spills 180 B, in the batch 1 KB, and is slower.
+template <int ST, bool MHD_F, bool CG>
+__device__ __forceinline__ void gather_node(const StepParams& p, const StepBuffers& b, uint32_t n, bool interior, int wp,
+                                            int wm, float (&v)[MHD_F ? 21 : 19], float (&l)[MHD_F ? 21 : 19])
+{
+    using T = typename Store<ST>::T;
+    if (interior) {
+        if constexpr (MHD_F) load_g_interior<ST, CG>(p, static_cast<const T*>(b.gsrc), n, wp, wm, v, l);
+        else load_f_interior<ST, CG>(p, static_cast<const T*>(b.fsrc), n, wp, wm, v, l);
+    } else {
+        uint32_t m = n;
+        asm volatile("" : "+r"(m));
+        const Geo g = make_geo(p, m);
+        if constexpr (MHD_F) load_g<ST, CG>(p, static_cast<const T*>(b.gsrc), g, v, l);
+        else load_f<ST, CG>(p, static_cast<const T*>(b.fsrc), g, v, l);
+    }
+}
+template <int ST, int MODE, bool CG>
+__device__ __forceinline__ void coupled_node2(const StepParams& p, const StepBuffers& b, uint32_t i, float (&acc)[7])
+{
+    if (!(i < p.N)) return;
+    const uint32_t n = i;
+    int wp = 0, wm = 0;
+    const bool interior = is_interior(p, n, wp, wm);
+    if (!interior && make_geo(p, n).solid) return;
+    float rho_inv, mx, my, mz;
+    const NodeIn<float> in = node_inputs<true, MODE_STEP>(p, b, n);
+    {
+        float d[19], dl[19];
+        gather_node<ST, false, CG>(p, b, n, interior, wp, wm, d, dl);
+        node_momentum<ST>(p, d, dl, rho_inv, mx, my, mz);
+    }
+    f_before_g();
+    {
+        float q[21], ql[21];
+        gather_node<ST, true, CG>(p, b, n, interior, wp, wm, q, ql);
+        induction_from_sources<ST>(p, b, n, in, rho_inv, mx, my, mz, q, ql);
+    }
+    const FieldOut fo{nullptr, nullptr, nullptr};
+    float d[19], dl[19], q[21], ql[21];
+    gather_node<ST, false, CG>(p, b, n, interior, wp, wm, d, dl);
+    node_from_sources<ST, false, MODE, false, 0>(p, b, fo, n, d, dl, q, ql, node_inputs<false, MODE, true>(p, b, n), acc);
+}
+
 // L2 prefetch for a step: the block b.pf_ahead positions later (one resident
 // wave of the kernel, so it starts about when this one ends) will gather
 // NODES consecutive nodes.  One thread per row asks L2 for that block's
@@ -1623,11 +1709,12 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
 // each side; with induction the 21 g rows (shifted like their D3Q7
 // direction) and the 3 rows of the lagged Lorentz force; the force rows; on
 // residual steps the 3 rows of the velocity snapshot.  Ranges are clamped to
-// their rows and trimmed to 16-byte boundaries.  Measured on the
+// their rows and trimmed to 16-byte boundaries.  with_f = false leaves the f
+// rows out (a cavity's blocks off the flow box).  Measured on the
 // 512 x 256 x 256 duct: BF16 paired step 0.4516 against 0.4829 ms, F32
 // one-node step 0.869 against 0.888 ms.
 template <int ST, int NODES, bool MHD, bool RESID>
-__device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBuffers& b)
+__device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBuffers& b, bool with_f = true)
 {
     using T = typename Store<ST>::T;
     constexpr int NG = MHD ? 21 : 0, NL = MHD ? 3 : 0;
@@ -1644,6 +1731,7 @@ __device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBu
     long long shift = 0, halo = 0;
     int r = t;
     if (r < 19) {
+        if (!with_f) return;
         row = reinterpret_cast<uintptr_t>(b.fsrc) + (uintptr_t)r * (uintptr_t)N * sizeof(T);
         esz = sizeof(T);
         shift = p.doff[r] - (long long)r * N;            // -(e_x + e_y nx + e_z nx ny)
@@ -1655,6 +1743,7 @@ __device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBu
         shift = p.doff[a] - (long long)a * N;
         halo = 1;
     } else if ((r -= NG) < NFC) {
+        if (!with_f) return;
         row = reinterpret_cast<uintptr_t>(b.fsrc) + (uintptr_t)19 * (uintptr_t)N * sizeof(T) +
               (uintptr_t)r * (uintptr_t)N * sizeof(__half);
         esz = sizeof(__half);
@@ -1695,8 +1784,11 @@ __device__ __forceinline__ void step_body(const StepParams& p, const StepBuffers
     if constexpr (MODE != MODE_FIELDS) advance_seed<ST>(b);
     // with induction only for F32 storage: coupled F32 step 0.1241 against
     // 0.1382 ms (half a wave ahead: 0.1200 ms), coupled BF16 step 0.0845
-    // against 0.0829 ms (half a wave ahead: 0.0841 ms)
-    if constexpr (MODE != MODE_FIELDS && (!MHD || ST == ST_F32))
+    // against 0.0829 ms (half a wave ahead: 0.0841 ms).  Fields: the 16-bit
+    // flow forms only (ten BF16 steps with fields on the 512 x 256 x 256 duct
+    // 5.012 -> 4.971 ms; the coupled F32 fields of 128^3 were slower with it)
+    constexpr bool PF = MODE == MODE_FIELDS ? !MHD && sizeof(typename Store<ST>::T) == 2 : !MHD || ST == ST_F32;
+    if constexpr (PF)
         prefetch_ahead<ST, STEP_THREADS, MHD, MODE == MODE_STEP_RESID>(p, b);
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -1708,8 +1800,8 @@ __device__ __forceinline__ void step_body(const StepParams& p, const StepBuffers
     // vs 0.842 ms; the coupled BF16 step keeps 80 registers with them: f
     // 1.2586 against 1.3008 ms on the 512 x 256 x 256 duct (the 21 g rows
     // from such bases too: 1.3385 ms)
-    scalar_node_step<ST, MHD, MODE, false, COLL == 0 && base_storage(ST) == ST_BF16 && MODE == MODE_STEP, false,
-                     COLL>(p, b, fo, i, acc);
+    scalar_node_step<ST, MHD, MODE, false, COLL == 0 && base_storage(ST) == ST_BF16 && MODE == MODE_STEP, COLL>(
+        p, b, fo, i, acc);
     if (MODE == MODE_STEP_RESID) block_partials<STEP_THREADS>(acc, b.partials);
 }
 
@@ -1748,9 +1840,7 @@ constexpr int step_dense_blocks()
 }
 
 // The coupled compensated step in two passes per thread (the batch's form):
-// pass 1 gathers f and g, runs the induction part and writes g~ and this
-// step's Lorentz force; pass 2 gathers f again (from L1 / L2) and runs the
-// flow update with F = F_ext + F_L.  The arithmetic and its order are the
+// see coupled_node2.  The arithmetic and its order are the
 // one-pass update's, so the result is bit for bit the same, but the
 // registers of the two parts are not live together: 172 registers in one
 // pass (one block of 256 per SM) against at most 128 here (F32C; the F32
@@ -1764,8 +1854,7 @@ __global__ void __launch_bounds__(STEP_THREADS, ST == ST_F32C ? 2 : 3)
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (MODE != MODE_STEP_RESID && !(i < p.N)) return;
-    coupled_induction_pass<ST, false>(p, b, i);
-    scalar_node_step<ST, false, MODE, false, false, true>(p, b, fo, i, acc);
+    coupled_node2<ST, MODE, false>(p, b, i, acc);
     if (MODE == MODE_STEP_RESID) block_partials<STEP_THREADS>(acc, b.partials);
 }
 
@@ -2132,8 +2221,11 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
             if (MODE != MODE_FIELDS && p.collision == 1) {
                 if constexpr (ST == ST_F32) cavity_kernel<ST, MHD, MODE, 1><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
             } else if (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS && p.variant == 0) {
-                if constexpr (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS)
+                if constexpr (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS) {
+                    static const long long wave = resident_wave(cavity_kernel_coupled2<ST, MODE>, STEP_THREADS);
+                    b.pf_ahead = (long long)grid > 4 * wave ? wave / 2 : 0;
                     cavity_kernel_coupled2<ST, MODE><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+                }
             } else {
                 cavity_kernel<ST, MHD, MODE, 0><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
             }

@@ -180,6 +180,17 @@ __device__ __forceinline__ void resident_update(const StepParams& p, const StepB
         const FieldOut fo{nullptr, nullptr, nullptr};
         float d[19], dl[19], q[21], ql[21];
         resident_load_f<ST>(p, fs, tab, stride, d, dl);
+        if constexpr (UNIT == RES_NODE2) {
+            float rho_inv, mx, my, mz;
+            const NodeIn<float> in = node_inputs<true, MODE_STEP>(p, b, i);
+            resident_load_g<ST>(p, static_cast<const T*>(b.gsrc), tab, stride, bounced, q, ql);
+            node_momentum<ST, false>(p, d, dl, rho_inv, mx, my, mz);
+            induction_from_sources<ST, false>(p, b, i, in, rho_inv, mx, my, mz, q, ql);
+            resident_load_f<ST>(p, fs, tab, stride, d, dl);
+            node_from_sources<ST, false, MODE, false, 0, false>(p, b, fo, i, d, dl, q, ql,
+                                                         node_inputs<false, MODE, true>(p, b, i), acc);
+            return;
+        }
         if constexpr (UNIT == RES_NODE1) {
             F1 v[19], vl[19], w[21], wl[21];
 #pragma unroll
@@ -189,14 +200,7 @@ __device__ __forceinline__ void resident_update(const StepParams& p, const StepB
             return;
         }
         if constexpr (MHD) resident_load_g<ST>(p, static_cast<const T*>(b.gsrc), tab, stride, bounced, q, ql);
-        if constexpr (UNIT == RES_NODE2) {
-            induction_from_sources<ST>(p, b, i, d, dl, q, ql);
-            resident_load_f<ST>(p, fs, tab, stride, d, dl);
-            node_from_sources<ST, false, MODE, false, 0>(p, b, fo, i, d, dl, q, ql,
-                                                         node_inputs<false, MODE, true>(p, b, i), acc);
-        } else {
-            node_from_sources<ST, MHD, MODE, false, 0>(p, b, fo, i, d, dl, q, ql, node_inputs<MHD, MODE>(p, b, i), acc);
-        }
+        node_from_sources<ST, MHD, MODE, false, 0, false>(p, b, fo, i, d, dl, q, ql, node_inputs<MHD, MODE>(p, b, i), acc);
     }
 }
 
