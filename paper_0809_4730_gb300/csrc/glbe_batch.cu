@@ -19,6 +19,7 @@
 // The block size and the number of resident blocks per SM are chosen by
 // glbe_batch_autotune, which times a few steps of each candidate on the batch
 // itself and then restores the rest state.
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -31,6 +32,10 @@ using namespace glbe;
 
 namespace {
 
+// Launch shape before any autotuning: as many blocks of 256 per SM as fit (16
+// ducts of 32 to 112 nodes an edge, F32C: 40.1 ms for 50 levels at one block
+// per SM, 31 ms at two).
+constexpr int BATCH_MOST_BLOCKS = 1 << 10;
 constexpr long long BARRIER_SPIN_LIMIT = 1ll << 26;   // default polls of ~64 ns: about 4 s
 
 struct BatchDomain {
@@ -394,7 +399,8 @@ glbe_status launch_batch(glbe_batch* b, long long nsteps, double tol, cudaStream
     if (s != GLBE_OK) return s;
     if (maxb < 1) return fail(GLBE_ERR_CUDA, "batch kernel cannot be resident (block %d)", b->block_threads);
     const int bps = b->blocks_per_sm < 1 ? 1 : (b->blocks_per_sm > maxb ? maxb : b->blocks_per_sm);
-    const unsigned grid = (unsigned)(bps * b->num_sms);
+    // no more blocks than tiles: the others would only wait at the barrier
+    const unsigned grid = std::min((unsigned)(bps * b->num_sms), std::max(ntiles, 1u));
     long long t0 = b->t, snap = b->snap_level;
     long long spin = b->spin_limit;
     int absent = b->absent_block;
@@ -471,7 +477,7 @@ glbe_status glbe_batch_init(const glbe_params* doms, int n, void* d_workspace, s
     off = align_up(off + sizeof(BatchState));
     b->d_dstate = reinterpret_cast<BatchDomainState*>(b->ws + off);
     b->block_threads = 256;
-    b->blocks_per_sm = 1;
+    b->blocks_per_sm = BATCH_MOST_BLOCKS;
     b->spin_limit = BARRIER_SPIN_LIMIT;
     b->absent_block = -1;
     int dev = 0;
