@@ -475,15 +475,10 @@ cudaError_t forward_step(const CtxView& v, const AdjLayout& L, const char* from,
     b.fdst = to + L.state_f;
     b.gsrc = v.prm.induction ? from + L.state_g : nullptr;
     b.gdst = v.prm.induction ? to + L.state_g : nullptr;
+    b.FLsrc = v.prm.induction ? reinterpret_cast<const float*>(from + L.state_FL) : nullptr;
     b.FL = v.prm.induction ? reinterpret_cast<float*>(to + L.state_FL) : nullptr;
     b.Ffield = v.Ffield;
     const FieldOut fo{nullptr, nullptr, nullptr};
-    if (v.prm.induction) {
-        // the step updates F_L in place: start the new slot from the old one
-        cudaError_t e = cudaMemcpyAsync(to + L.state_FL, from + L.state_FL, 3 * v.N * sizeof(float),
-                                        cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-    }
     if (v.prm.storage == GLBE_F32) return launch_step_t<ST_F32>(v.prm.induction, MODE_STEP, v.sp, b, fo, st, nullptr);
     return launch_step_t<ST_F32C>(v.prm.induction, MODE_STEP, v.sp, b, fo, st, nullptr);
 }
@@ -664,13 +659,11 @@ glbe_status glbe_adjoint_unrolled(glbe_ctx* ctx, const float* d_w, long nsteps, 
     // reverse sweep, one segment of up to K levels at a time
     for (long i = L.ncp - 1; i >= 0; --i) {
         const long len = (i + 1) * K <= nsteps ? K : nsteps - i * K;
-        ADJ_CUDA(cudaMemcpyAsync(seg, cp + (size_t)i * L.state_bytes, L.state_bytes, cudaMemcpyDeviceToDevice, st),
-                 "restore checkpoint");
-        for (long j = 0; j + 1 < len; ++j)
-            ADJ_CUDA(forward_step(v, L, seg + (size_t)j * L.state_bytes, seg + (size_t)(j + 1) * L.state_bytes, st),
-                     "recompute step");
+        // level 0 of the segment is its checkpoint, read where it lies
+        auto level = [&](long j) { return j == 0 ? cp + (size_t)i * L.state_bytes : seg + (size_t)j * L.state_bytes; };
+        for (long j = 0; j + 1 < len; ++j) ADJ_CUDA(forward_step(v, L, level(j), level(j + 1), st), "recompute step");
         for (long j = len - 1; j >= 0; --j) {
-            set_forward(a, v, L, seg + (size_t)j * L.state_bytes);
+            set_forward(a, v, L, level(j));
             a.lam_in = lam[cur];
             a.lam_out = lam[cur ^ 1];
             ADJ_CUDA(launch_adjoint(v.prm.storage, v.prm.induction, false, v.sp, a, st, nullptr), "adjoint step");

@@ -393,6 +393,7 @@ StepBuffers buffers_for(glbe_ctx* c, long t)
     b.fdst = c->f[s ^ 1];
     b.gsrc = c->prm.induction ? c->g[s] : nullptr;
     b.gdst = c->prm.induction ? c->g[s ^ 1] : nullptr;
+    b.FLsrc = c->FL;
     b.FL = c->FL;
     b.Ffield = c->Ffield;
     b.usnap = c->usnap;

@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(BT, 512 / BT) batch_kernel(const BatchDomain* 
                 b.fdst = D.f[par ^ 1];
                 b.gsrc = D.g[par];
                 b.gdst = D.g[par ^ 1];
+                b.FLsrc = D.FL;
                 b.FL = D.FL;
                 b.usnap = D.usnap;
                 b.snap_lo = 1;
@@ -676,6 +677,7 @@ glbe_status glbe_batch_fields(glbe_batch* b, int d, float* d_rho, float* d_u, fl
     const int par = (int)(lvl & 1);
     sb.fsrc = D.f[par];
     sb.gsrc = D.g[par];
+    sb.FLsrc = D.FL;
     sb.FL = D.FL;
     sb.usnap = D.usnap;
     const FieldOut fo{d_rho, d_u, D.mhd ? d_B : nullptr};

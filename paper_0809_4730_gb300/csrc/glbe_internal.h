@@ -83,7 +83,8 @@ struct StepBuffers {
     void* fdst;
     const void* gsrc;
     void* gdst;
-    float* FL;            // [3][N] Lorentz force of the previous step (in place)
+    const float* FLsrc;   // [3][N] Lorentz force of the previous step
+    float* FL;            // [3][N] this step's Lorentz force (FLsrc itself: in place)
     const float* Ffield;  // [force_ncomp][N] or null
     float* usnap;         // [3][N] velocity snapshot of the last residual level; with snap_lo
                           // [6][N], rows 3..5 the low parts of u (double-float snapshot)

@@ -1327,9 +1327,9 @@ __device__ __forceinline__ NodeIn<float> node_inputs(const StepParams& p, const 
     NodeIn<float> in;
     in.FLx = in.FLy = in.FLz = 0.f;
     if (MHD) {
-        in.FLx = b.FL[n];
-        in.FLy = b.FL[N + n];
-        in.FLz = b.FL[2 * N + n];
+        in.FLx = b.FLsrc[n];
+        in.FLy = b.FLsrc[N + n];
+        in.FLz = b.FLsrc[2 * N + n];
     }
     in.Fx = p.F[0];
     in.Fy = p.F[1];
@@ -1366,9 +1366,9 @@ __device__ __forceinline__ NodeIn<V> pair_inputs(const StepParams& p, const Step
     NodeIn<V> in;
     in.FLx = in.FLy = in.FLz = V(0.f);
     if (MHD) {
-        ldv(b.FL + n0, in.FLx);
-        ldv(b.FL + N + n0, in.FLy);
-        ldv(b.FL + 2 * N + n0, in.FLz);
+        ldv(b.FLsrc + n0, in.FLx);
+        ldv(b.FLsrc + N + n0, in.FLy);
+        ldv(b.FLsrc + 2 * N + n0, in.FLz);
     }
     in.Fx = V(p.F[0]);
     in.Fy = V(p.F[1]);
@@ -1757,7 +1757,7 @@ __device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBu
         shift = p.doff[a] - (long long)a * N;
         halo = 1;
     } else if ((r -= NGC) < NL) {
-        row = reinterpret_cast<uintptr_t>(b.FL) + (uintptr_t)r * (uintptr_t)N * sizeof(float);
+        row = reinterpret_cast<uintptr_t>(b.FLsrc) + (uintptr_t)r * (uintptr_t)N * sizeof(float);
         esz = sizeof(float);
     } else if ((r -= NL) < 3) {
         if (r >= p.force_ncomp || b.Ffield == nullptr) return;

@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
     else if (threadIdx.x == 0) gen = *(volatile unsigned*)(m.bar + 1);
     const bool writer = blockIdx.x == G - 1;    // the last block has no more tiles than any other
     StepBuffers b{};
+    b.FLsrc = m.FL;
     b.FL = m.FL;
     b.Ffield = m.Ffield;
     b.usnap = m.usnap;
