@@ -6,16 +6,18 @@
 // most of it the launch itself, kernel prologue, geometry and the latency of
 // one gather.  Resident, a step takes (us, launched before -> resident):
 //                 F32 flow      F32 coupled   F32C flow     F32C coupled
-//   4 x 32 x 4    8.5 -> 2.2    8.5 -> 2.6    8.5 -> 2.3    10.0 -> 3.5
+//   4 x 32 x 4    8.5 -> 1.9    8.5 -> 2.6    8.5 -> 1.6    10.0 -> 3.5
 //   64 x 64 x 8   8.7 -> 3.9    8.7 -> 4.6    8.5 -> 4.0    10.5 -> 5.7
 //   40^3          8.8 -> 4.4   10.8 -> 6.4   10.6 -> 5.6    14.6 -> 9.0
-//   64^3         13.2 -> 9.5   21.5 -> 17.5  17.7 -> 15.4   37.9 -> 31
+//   64^3         13.2 -> 9.4   21.5 -> 17.5  17.7 -> 15.2   37.9 -> 30.4
 // (launched: with the reduction of glbe_residual.cuh).  The line lies where
 // the tables crowd out the gathers' L1 (RES_TABLES_FLOW, RES_TABLES_MHD):
 // 72^3 coupled marched 32.7 us a step with 205 KB of tables on an SM, 29.5
 // launched (F32C 56.3 and 52.7).  The node update is the step kernels'
 // (node_from_sources, pair_from_sources), so the states are theirs bit for bit.
 #pragma once
+#include <type_traits>
+
 #include "glbe_resident_common.cuh"
 
 namespace glbe {
@@ -157,7 +159,7 @@ __device__ __forceinline__ void resident_load_g(const StepParams& p, const typen
 
 // What a thread updates: a pair of nodes, as step_pair_kernel (flow, where
 // pair_eligible says so), else one node, as step_kernel; a coupled node in one
-// pass or (RES_NODE2) in two (see coupled_induction_pass).  Each is that
+// pass or (RES_NODE2) in two (see coupled_node2).  Each is that
 // kernel's arithmetic, so a march gives the same bits whichever launches it.
 // RES_NODE1 is one node in the pair's arithmetic: on grids of no more than a
 // tile per block a step is a chain of latencies, and a thread that gathers two
@@ -322,28 +324,282 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
     }
 }
 
+// The cluster form of the flow lattice (up to 16 x 256 nodes): it lives in the
+// shared memory of 16 blocks, both population buffers, forces and snapshot, and
+// a gather is a load from distributed shared memory: the tables hold the
+// sources' addresses in the cluster's window.  A level then costs two
+// shared-memory latencies and a cluster barrier instead of two trips to L2
+// (4 x 32 x 4: F32 2.16 us a step through L2, 1.89 here; F32C 2.4 and 1.6).  The state is read
+// from the workspace at the start and left there at the end.
+template <class T>
+__device__ __forceinline__ float ld_cluster(uint32_t addr)
+{
+    if constexpr (sizeof(T) == 4) {
+        float v;
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+        return v;
+    } else {
+        unsigned short u;
+        asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(u) : "r"(addr));
+        if constexpr (std::is_same<T, __half>::value) return __half2float(__ushort_as_half(u));
+        else return __uint_as_float((unsigned)u << 16);
+    }
+}
+__device__ __forceinline__ uint32_t cluster_address(uint32_t local, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+    return a;
+}
+
+// Inputs of the node in column tid (see node_inputs): b's force field, lagged
+// force and snapshot are columns of shared memory here.  Volatile loads, like
+// the gathers': with plain ones the compiler forms what the two kinds of levels
+// have in common ahead of the branch between them (the product of the half
+// force, say) and then cannot contract it with what follows, as the launched
+// steps do: a unit in the last place, rarely, but not the same bits.
+template <class V, int MODE>
+__device__ __forceinline__ NodeIn<V> cluster_inputs(const StepParams& p, const StepBuffers& b, int tid)
+{
+    const int N = (int)p.N;
+    const volatile float *F = b.Ffield, *us = b.usnap;
+    NodeIn<V> in;
+    in.FLx = in.FLy = in.FLz = V(0.f);
+    in.Fx = V(p.F[0]);
+    in.Fy = V(p.F[1]);
+    in.Fz = V(p.F[2]);
+    if (p.force_ncomp >= 1) in.Fx += V(F[tid]);
+    if (p.force_ncomp == 3) {
+        in.Fy += V(F[N + tid]);
+        in.Fz += V(F[2 * N + tid]);
+    }
+    in.us0 = in.us1 = in.us2 = V(0.f);
+    in.ul0 = in.ul1 = in.ul2 = V(0.f);
+    if (MODE == MODE_STEP_RESID && b.have_snap) {
+        in.us0 = V(us[tid]);
+        in.us1 = V(us[N + tid]);
+        in.us2 = V(us[2 * N + tid]);
+        if (b.snap_lo) {
+            in.ul0 = V(us[3 * N + tid]);
+            in.ul1 = V(us[4 * N + tid]);
+            in.ul2 = V(us[5 * N + tid]);
+        }
+    }
+    return in;
+}
+
+// Bytes of a block's shared memory and where its parts lie.
+struct ClusterLayout {
+    unsigned f, flo, fstep, F, snap, tab, tablo, total;
+};
+__host__ __device__ inline ClusterLayout cluster_layout(int T, bool comp, int BT)
+{
+    ClusterLayout L{};
+    unsigned off = 0;
+    const unsigned lo = comp ? 2u : 0u, b = (unsigned)BT;
+    L.f = off;
+    L.flo = off + 19u * b * T;
+    L.fstep = 19u * b * (T + lo);
+    off += 2 * L.fstep;
+    L.F = off;
+    off += 3u * b * 4u;
+    L.snap = off;
+    off += 6u * b * 4u;
+    L.tab = off;
+    off += RES_ROWS * b * 4u;
+    L.tablo = off;
+    if (comp) off += 19u * b * 4u;
+    L.total = off;
+    return L;
+}
+
+template <int ST, bool PAIR>
+__global__ void __launch_bounds__(RES_THREADS, 1) resident_cluster_kernel(const StepParams p, const ResidentMarch m)
+{
+    using S = Store<ST>;
+    using T = typename S::T;
+    constexpr bool COMP = S::COMP;
+    extern __shared__ __align__(16) char sm[];
+    __shared__ float wsum[RES_THREADS / 32][RES_SUMS];
+    __shared__ double bsum[RES_SUMS];
+    __shared__ double part[RES_SUMS * RES_CLUSTER];
+    __shared__ double tot[RES_SUMS];
+    __shared__ int verdict;
+    const int BT = blockDim.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (m.solve && *(volatile int*)m.out.stop) return;   // converged in an earlier launch
+    const ClusterLayout L = cluster_layout(sizeof(T), COMP, BT);
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+    const uint32_t n = blockIdx.x * BT + tid;
+    const bool inb = n < p.N;
+    const size_t N = p.N;
+    uint32_t* tab = reinterpret_cast<uint32_t*>(sm + L.tab) + tid;
+    uint32_t* tablo = reinterpret_cast<uint32_t*>(sm + L.tablo) + tid;
+    resident_slots(p, n, tab, BT);
+    const unsigned flags = tab[19 * BT];
+    if (flags != RES_SKIP) {
+        for (int a = 0; a < 19; ++a) {
+            const uint32_t s = tab[a * BT], row = s / p.N, src = s - row * p.N, rank = src / BT;
+            const uint32_t k = row * BT + (src - rank * BT);
+            tab[a * BT] = cluster_address(base + L.f + k * (uint32_t)sizeof(T), rank);
+            if constexpr (COMP) tablo[a * BT] = cluster_address(base + L.flo + k * 2u, rank);
+        }
+    }
+    // the state of level t0; of a node that is not updated both buffers, since a
+    // ghost plane's is gathered from (a solid node's never)
+    const int par0 = m.phase & 1;
+    float* const F = reinterpret_cast<float*>(sm + L.F);
+    float* const snapc = reinterpret_cast<float*>(sm + L.snap);
+    auto rows = [&](int h, bool load) {
+        T* g = static_cast<T*>(m.f[h]);
+        T* c = reinterpret_cast<T*>(sm + L.f + h * L.fstep);
+        for (int a = 0; a < 19; ++a) {
+            if (load) c[a * BT + tid] = g[a * N + n];
+            else g[a * N + n] = c[a * BT + tid];
+        }
+        if constexpr (COMP) {
+            __half* gl = reinterpret_cast<__half*>(g + 19 * N);
+            __half* cl = reinterpret_cast<__half*>(sm + L.flo + h * L.fstep);
+            for (int a = 0; a < 19; ++a) {
+                if (load) cl[a * BT + tid] = gl[a * N + n];
+                else gl[a * N + n] = cl[a * BT + tid];
+            }
+        }
+    };
+    if (inb) {
+        for (int k = 0; k < (flags == RES_SKIP ? 2 : 1); ++k) rows(par0 ^ k, true);
+        for (int k = 0; k < p.force_ncomp; ++k) F[k * BT + tid] = m.Ffield[k * N + n];
+        for (int k = 0; k < (m.snap_lo ? 6 : 3); ++k) snapc[k * BT + tid] = m.usnap[k * N + n];
+    }
+    cluster_level_barrier();
+    StepParams q = p;
+    q.N = (uint32_t)BT;                         // the columns' stride in shared memory
+    StepBuffers b{};
+    b.Ffield = F;
+    b.usnap = snapc;
+    b.snap_lo = m.snap_lo;
+    const FieldOut fo{nullptr, nullptr, nullptr};
+    const bool writer = blockIdx.x == G - 1;
+    bool snap = m.have_snap != 0;               // the snapshot is of the previous residual level
+    int par = par0;
+    for (int s = 0, phase = m.phase; s < m.nsteps; ++s, phase = phase == 9 ? 0 : phase + 1) {
+        const bool resid = phase == 0;
+        b.fdst = sm + L.f + (par ^ 1) * L.fstep;
+        b.have_snap = snap ? 1 : 0;
+        float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (flags != RES_SKIP) {
+            auto update = [&](auto mode) {
+                constexpr int MODE = decltype(mode)::value;
+                float d[19], dl[19], v[21], vl[21];
+                const uint32_t df = par * L.fstep;
+#pragma unroll
+                for (int a = 0; a < 19; ++a) {
+                    d[a] = unscale<ST>(p, ld_cluster<T>(tab[a * BT] + df));
+                    if constexpr (COMP) dl[a] = ld_cluster<__half>(tablo[a * BT] + df) * LO_INV;
+                }
+                if constexpr (PAIR) {
+                    F1 w[19], wl[19], z[21], zl[21];
+#pragma unroll
+                    for (int a = 0; a < 19; ++a) w[a] = F1(d[a]);
+                    pair_from_sources<ST, false, MODE, false, F1>(q, b, tid, w, wl, z, zl,
+                                                                  cluster_inputs<F1, MODE>(q, b, tid), acc);
+                } else {
+                    node_from_sources<ST, false, MODE, false, 0, false>(q, b, fo, tid, d, dl, v, vl,
+                                                                      cluster_inputs<float, MODE>(q, b, tid), acc);
+                }
+            };
+            if (resid) update(std::integral_constant<int, MODE_STEP_RESID>{});
+            else update(std::integral_constant<int, MODE_STEP>{});
+        }
+        if (resid && snap) {
+#pragma unroll
+            for (int r = 0; r < RES_SUMS; ++r) {
+                const float x = warp_sum(acc[r]);
+                if (lane == 0) wsum[warp][r] = x;
+            }
+            __syncthreads();
+            if (tid < RES_SUMS) {
+                float x = 0.f;
+                for (int w = 0; w < BT / 32; ++w) x += wsum[w][tid];
+                bsum[tid] = (double)x;
+            }
+            __syncthreads();
+            // every block's sums into every block's shared memory
+            auto cl = cooperative_groups::this_cluster();
+            for (int i = tid; i < RES_SUMS * G; i += BT)
+                cl.map_shared_rank(part, (unsigned)(i / RES_SUMS))[(i % RES_SUMS) * RES_CLUSTER + blockIdx.x] =
+                    bsum[i % RES_SUMS];
+        }
+        cluster_level_barrier();
+        par ^= 1;
+        if (!resid) continue;
+        if (snap && (m.solve || writer)) {
+            // a solve's blocks all take the decision, from the same sums in the same order
+            for (int k = warp; k < RES_SUMS; k += BT / 32) {
+                const double x = warp_sum_all(lane < G ? part[k * RES_CLUSTER + lane] : 0.0);
+                if (lane == 0) tot[k] = x;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                verdict = m.solve && resident_stops(m.tol, tot);
+                if (writer && !*m.out.stop) write_record(m.out, tot, *m.out.t_dev);
+            }
+            __syncthreads();
+            if (verdict) break;                 // the state is the one after this level, in every block
+        } else if (!snap && writer && tid == 0) {
+            *m.out.t_dev = m.t0 + s + 10;
+        }
+        snap = true;
+    }
+    if (inb && flags != RES_SKIP) {
+        rows(par, false);
+        for (int k = 0; k < (m.snap_lo ? 6 : 3); ++k) m.usnap[k * N + n] = snapc[k * BT + tid];
+    }
+}
+
+// The kernel of the cluster form.  A coupled lattice goes through L2: from
+// shared memory its update came out a unit in the last place off now and then
+// (the compiler contracted it differently there).
+template <int ST, bool MHD, bool PAIR>
+constexpr auto resident_cluster_form()
+{
+    if constexpr (MHD) return resident_kernel<ST, true, false, false, true>;
+    else return resident_cluster_kernel<ST, PAIR>;
+}
+template <int ST, bool MHD>
+unsigned resident_cluster_bytes(int threads)
+{
+    return MHD ? (unsigned)(RES_ROWS * threads * sizeof(uint32_t))
+               : cluster_layout(sizeof(typename Store<ST>::T), Store<ST>::COMP, threads).total;
+}
+
 template <int ST, bool MHD, bool PAIR>
 cudaError_t resident_plan_t(uint32_t N, ResidentPlan* out)
 {
     constexpr size_t tile = (size_t)RES_ROWS * RES_THREADS * sizeof(uint32_t);
-    auto* cluster = resident_kernel<ST, MHD, PAIR, false, true>;
+    constexpr auto cluster = resident_cluster_form<ST, MHD, PAIR>();
     auto* free_form = resident_kernel<ST, MHD, PAIR, false, false>;
     auto* dense = resident_kernel<ST, MHD, PAIR, true, false>;
+    const unsigned most = resident_cluster_bytes<ST, MHD>(RES_THREADS);
     static const ResidentOcc of = resident_occupancy(free_form, tile), od = resident_occupancy(dense, tile);
     static const bool fits = [&] {
         cudaFuncSetAttribute(cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return resident_cluster_fits(cluster, tile);
+        cudaFuncSetAttribute(cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        return resident_cluster_fits(cluster, most);
     }();
-    const cudaError_t e = resident_plan_of(cluster, free_form, dense, N, PAIR ? N >> 1 : N, RES_ROWS,
-                                           MHD ? RES_TABLES_MHD : RES_TABLES_FLOW, of, od, fits, out);
+    cudaError_t e = resident_plan_of(cluster, free_form, dense, N, PAIR ? N >> 1 : N, RES_ROWS,
+                                     MHD ? RES_TABLES_MHD : RES_TABLES_FLOW, of, od, fits, out);
     out->pair = PAIR ? 1 : 0;
+    if (e == cudaSuccess && out->form == 1) {
+        out->smem = resident_cluster_bytes<ST, MHD>(out->threads);
+        e = cudaFuncSetAttribute(cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    }
     return e;
 }
 
 template <int ST, bool MHD, bool PAIR>
 cudaError_t resident_march_t(const StepParams& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
 {
-    if (pl.form == 1) return resident_launch(resident_kernel<ST, MHD, PAIR, false, true>, pl, st, p, m);
+    if (pl.form == 1) return resident_launch(resident_cluster_form<ST, MHD, PAIR>(), pl, st, p, m);
     if (pl.form == 2) return resident_launch(resident_kernel<ST, MHD, PAIR, false, false>, pl, st, p, m);
     return resident_launch(resident_kernel<ST, MHD, PAIR, true, false>, pl, st, p, m);
 }

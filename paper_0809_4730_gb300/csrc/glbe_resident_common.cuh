@@ -158,8 +158,8 @@ inline bool resident_grid_plan(const ResidentOcc& occ, uint32_t units, int sms, 
 // block (registers unbounded), several tiles a block (held to the register
 // budget of the launched steps).  units_dense: updates of the dense form.
 // The attributes set are the device's: the same values whoever sets them.
-template <class K>
-cudaError_t resident_plan_of(K cluster, K free_form, K dense, uint32_t N, uint32_t units_dense, int rows,
+template <class C, class K>
+cudaError_t resident_plan_of(C cluster, K free_form, K dense, uint32_t N, uint32_t units_dense, int rows,
                              size_t table_bytes, const ResidentOcc& occ_free, const ResidentOcc& occ_dense, bool cluster_fits,
                              ResidentPlan* out)
 {
