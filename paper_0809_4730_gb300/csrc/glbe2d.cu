@@ -877,6 +877,8 @@ __device__ __forceinline__ void load_snap2(const P2& p, const B2& b, int n, floa
 template <int ST, bool MHD, int MODE>
 __device__ __forceinline__ void step2d_body(const P2& p, const B2& b, const Out2& o)
 {
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop && *b.stop) return;   // the march converged in an earlier launch of this chunk
     if constexpr (MODE != M2_FIELDS) prefetch2d<ST, MHD, MODE == M2_RESID>(p, b);
     const int n = blockIdx.x * T2D + threadIdx.x;
@@ -1305,6 +1307,8 @@ struct DirG {    // the 10 rows of g: component j = r / 5, direction r % 5
 template <int ST, bool MHD, int MODE>
 __global__ void __launch_bounds__(T2D) step2d_pair_kernel(const P2 p, const B2 b)
 {
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop && *b.stop) return;
     const int lane = threadIdx.x & 31;
     const int n0 = 2 * (blockIdx.x * T2D + threadIdx.x);
@@ -1688,17 +1692,18 @@ cudaError_t launch2_t(glbe2d_ctx* c, int mode, const B2& b_in, const Out2& o, cu
     const bool mhd = c->prm.induction;
     const unsigned nb = c->blocks;
     B2 b = b_in;
+    cudaError_t e = cudaSuccess;
     if constexpr (ST == GLBE_F32 || ST == GLBE_BF16) {
         if (c->pair && mode != M2_FIELDS) {
             const unsigned pb = c->pair_blocks;
             if (mode == M2_STEP) {
-                if (mhd) step2d_pair_kernel<ST, true, M2_STEP><<<pb, T2D, 0, st>>>(c->p, b);
-                else step2d_pair_kernel<ST, false, M2_STEP><<<pb, T2D, 0, st>>>(c->p, b);
+                if (mhd) e = launch_overlapped(step2d_pair_kernel<ST, true, M2_STEP>, pb, T2D, st, c->p, b);
+                else e = launch_overlapped(step2d_pair_kernel<ST, false, M2_STEP>, pb, T2D, st, c->p, b);
             } else {
-                if (mhd) step2d_pair_kernel<ST, true, M2_RESID><<<pb, T2D, 0, st>>>(c->p, b);
-                else step2d_pair_kernel<ST, false, M2_RESID><<<pb, T2D, 0, st>>>(c->p, b);
+                if (mhd) e = launch_overlapped(step2d_pair_kernel<ST, true, M2_RESID>, pb, T2D, st, c->p, b);
+                else e = launch_overlapped(step2d_pair_kernel<ST, false, M2_RESID>, pb, T2D, st, c->p, b);
             }
-            return cudaGetLastError();
+            return e;
         }
     }
     if (mode == M2_STEP) {
@@ -1707,43 +1712,43 @@ cudaError_t launch2_t(glbe2d_ctx* c, int mode, const B2& b_in, const Out2& o, cu
             if constexpr (MBM > 0) {
                 if (c->prm.variant == 0) {
                     b.pf_ahead = prefetch_distance<ST, true>(step2d_kernel_dense<ST, true, MBM>, nb);
-                    step2d_kernel_dense<ST, true, MBM><<<nb, T2D, 0, st>>>(c->p, b, o);
-                    return cudaGetLastError();
+                    e = launch_overlapped(step2d_kernel_dense<ST, true, MBM>, nb, T2D, st, c->p, b, o);
+                    return e;
                 }
             }
             b.pf_ahead = prefetch_distance<ST, true>(step2d_kernel<ST, true, M2_STEP>, nb);
-            step2d_kernel<ST, true, M2_STEP><<<nb, T2D, 0, st>>>(c->p, b, o);
+            e = launch_overlapped(step2d_kernel<ST, true, M2_STEP>, nb, T2D, st, c->p, b, o);
         } else {
             if constexpr (MBF > 0) {
                 if (c->prm.variant == 0) {
                     b.pf_ahead = prefetch_distance<ST, false>(step2d_kernel_dense<ST, false, MBF>, nb);
-                    step2d_kernel_dense<ST, false, MBF><<<nb, T2D, 0, st>>>(c->p, b, o);
-                    return cudaGetLastError();
+                    e = launch_overlapped(step2d_kernel_dense<ST, false, MBF>, nb, T2D, st, c->p, b, o);
+                    return e;
                 }
             }
             b.pf_ahead = prefetch_distance<ST, false>(step2d_kernel<ST, false, M2_STEP>, nb);
-            step2d_kernel<ST, false, M2_STEP><<<nb, T2D, 0, st>>>(c->p, b, o);
+            e = launch_overlapped(step2d_kernel<ST, false, M2_STEP>, nb, T2D, st, c->p, b, o);
         }
     } else if (mode == M2_RESID) {
         if (mhd) {
             if constexpr (ST == GLBE_F32) {
                 if (c->prm.variant == 0) {
                     b.pf_ahead = prefetch_distance<ST, true>(step2d_kernel_dense_resid<ST, 4>, nb);
-                    step2d_kernel_dense_resid<ST, 4><<<nb, T2D, 0, st>>>(c->p, b, o);
-                    return cudaGetLastError();
+                    e = launch_overlapped(step2d_kernel_dense_resid<ST, 4>, nb, T2D, st, c->p, b, o);
+                    return e;
                 }
             }
             b.pf_ahead = prefetch_distance<ST, true>(step2d_kernel<ST, true, M2_RESID>, nb);
-            step2d_kernel<ST, true, M2_RESID><<<nb, T2D, 0, st>>>(c->p, b, o);
+            e = launch_overlapped(step2d_kernel<ST, true, M2_RESID>, nb, T2D, st, c->p, b, o);
         } else {
             b.pf_ahead = prefetch_distance<ST, false>(step2d_kernel<ST, false, M2_RESID>, nb);
-            step2d_kernel<ST, false, M2_RESID><<<nb, T2D, 0, st>>>(c->p, b, o);
+            e = launch_overlapped(step2d_kernel<ST, false, M2_RESID>, nb, T2D, st, c->p, b, o);
         }
     } else {
-        if (mhd) step2d_kernel<ST, true, M2_FIELDS><<<nb, T2D, 0, st>>>(c->p, b, o);
-        else step2d_kernel<ST, false, M2_FIELDS><<<nb, T2D, 0, st>>>(c->p, b, o);
+        if (mhd) e = launch_overlapped(step2d_kernel<ST, true, M2_FIELDS>, nb, T2D, st, c->p, b, o);
+        else e = launch_overlapped(step2d_kernel<ST, false, M2_FIELDS>, nb, T2D, st, c->p, b, o);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch2(glbe2d_ctx* c, int mode, const B2& b, const Out2& o, cudaStream_t st)

@@ -86,6 +86,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 4) adjoint_kernel(const StepParam
 {
     using S = Store<ST>;
     using T = typename S::T;
+    grid_dependency_release();
+    grid_dependency_wait();
     if (a.stop != nullptr && *a.stop) return;
     const uint32_t i = blockIdx.x * ADJ_THREADS + threadIdx.x;
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -331,16 +333,17 @@ template <int ST, bool MHD>
 cudaError_t launch_adj2(bool resid, const StepParams& p, const AdjArgs& a, cudaStream_t st, unsigned* nblocks)
 {
     const unsigned grid = (unsigned)(((size_t)p.N + ADJ_THREADS - 1) / ADJ_THREADS);
+    cudaError_t e;
     if (a.lin) {
         // no state gather: one instantiation serves both storage forms
-        if (resid) adjoint_kernel<ST_F32, MHD, true, true><<<grid, ADJ_THREADS, 0, st>>>(p, a);
-        else adjoint_kernel<ST_F32, MHD, false, true><<<grid, ADJ_THREADS, 0, st>>>(p, a);
+        if (resid) e = launch_overlapped(adjoint_kernel<ST_F32, MHD, true, true>, grid, ADJ_THREADS, st, p, a);
+        else e = launch_overlapped(adjoint_kernel<ST_F32, MHD, false, true>, grid, ADJ_THREADS, st, p, a);
     } else {
-        if (resid) adjoint_kernel<ST, MHD, true, false><<<grid, ADJ_THREADS, 0, st>>>(p, a);
-        else adjoint_kernel<ST, MHD, false, false><<<grid, ADJ_THREADS, 0, st>>>(p, a);
+        if (resid) e = launch_overlapped(adjoint_kernel<ST, MHD, true, false>, grid, ADJ_THREADS, st, p, a);
+        else e = launch_overlapped(adjoint_kernel<ST, MHD, false, false>, grid, ADJ_THREADS, st, p, a);
     }
     if (nblocks) *nblocks = grid;
-    return cudaGetLastError();
+    return e;
 }
 
 template <int ST, bool MHD>

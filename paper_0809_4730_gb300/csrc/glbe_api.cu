@@ -287,6 +287,8 @@ constexpr int FIN_THREADS = 256;
 __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(double* __restrict__ partials, unsigned nblocks,
                                                                const RecordOut out)
 {
+    grid_dependency_release();
+    grid_dependency_wait();
     if (*out.stop) return;   // a solve already converged: the chunk's remaining work is skipped
     __shared__ double tot[RES_SUMS];
     __shared__ int last;
@@ -544,8 +546,8 @@ cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, lo
                             const double* tol, cudaStream_t st)
 {
     const RecordOut out{record, hist, hist_count, hist_cap, t_dev, stop, tol, mass0};
-    finalize_kernel<<<(nblocks + FIN_CHUNK - 1) / FIN_CHUNK, FIN_THREADS, 0, st>>>(partials, nblocks, out);
-    return cudaGetLastError();
+    return launch_overlapped(finalize_kernel, (nblocks + FIN_CHUNK - 1) / FIN_CHUNK, FIN_THREADS, st, partials, nblocks,
+                             out);
 }
 }  // namespace glbe
 

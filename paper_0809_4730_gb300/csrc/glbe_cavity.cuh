@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(STEP_THREADS) cavity_kernel(const StepParams p
                                                               const FieldOut fo)
 {
     using T = typename Store<ST>::T;
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop != nullptr && *b.stop) return;
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -223,6 +225,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 3) cavity_kernel_coupled2(const 
 {
     using T = typename Store<ST>::T;
     constexpr bool PRECISE = (ST == ST_F32 || ST == ST_F32C);
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop != nullptr && *b.stop) return;
     prefetch_ahead<ST, STEP_THREADS, true, MODE == MODE_STEP_RESID>(p, b, box_ahead(p, b));
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;

@@ -241,6 +241,34 @@ inline long long fluid_nodes(const glbe_params* p)
 }
 StepParams make_step_params(const glbe_params* p);
 
+// Launches a kernel that may begin while the stream's previous kernel is still
+// ending (programmatic dependent launch): it calls grid_dependency_wait()
+// before it reads or writes anything, and the previous kernel, if it is one of
+// these, lets it begin once all its own blocks have started
+// (grid_dependency_release(); so no block waits for room that a waiting one
+// holds).  What is hidden is the launch and the first blocks' set-up, 2 to 4 us
+// a step: ten coupled F32 steps on 128^3 with fields 1297 -> 1263 us, twenty of
+// the 98^3 MHD cavity 2135 -> 2086 us, a 40-step transient's gradient on 64^3
+// 4298 -> 4083 us.
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t st, const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
 // What another translation unit (the adjoint) needs of a context: its
 // parameters and the buffers of the current time level t (the populations the
 // next step gathers from, the lagged Lorentz force, the force field).

@@ -1780,6 +1780,8 @@ __device__ __forceinline__ void prefetch_ahead(const StepParams& p, const StepBu
 template <int ST, bool MHD, int MODE, int COLL = 0>
 __device__ __forceinline__ void step_body(const StepParams& p, const StepBuffers& b, const FieldOut& fo)
 {
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop != nullptr && *b.stop) return;   // converged solve: remaining steps of the chunk are skipped
     if constexpr (MODE != MODE_FIELDS) advance_seed<ST>(b);
     // with induction only for F32 storage: coupled F32 step 0.1241 against
@@ -1849,6 +1851,8 @@ template <int ST, int MODE>
 __global__ void __launch_bounds__(STEP_THREADS, ST == ST_F32C ? 2 : 3)
     step_kernel_coupled2(const StepParams p, const StepBuffers b, const FieldOut fo)
 {
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop != nullptr && *b.stop) return;
     prefetch_ahead<ST, STEP_THREADS, true, MODE == MODE_STEP_RESID>(p, b);
     const uint32_t i = blockIdx.x * STEP_THREADS + threadIdx.x;
@@ -1987,6 +1991,8 @@ __device__ __forceinline__ void pair_step_body(const StepParams& p, const StepBu
 {
     using S = Store<ST>;
     using T = typename S::T;
+    grid_dependency_release();
+    grid_dependency_wait();
     if (b.stop != nullptr && *b.stop) return;
     advance_seed<ST>(b);
     if constexpr (!MHD && !S::COMP) prefetch_ahead<ST, 2 * PAIR_THREADS, false, MODE == MODE_STEP_RESID>(p, b);
@@ -2214,32 +2220,33 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
                         unsigned* nblocks)
 {
     StepBuffers b = with_dir_bases<ST>(p, b_in);
+    cudaError_t e = cudaSuccess;
     b.pf_ahead = 0;
     if constexpr (ST == ST_F32 || ST == ST_F32C || ST == ST_BF16) {
         if (p.cavity) {   // fluid box and / or moving lid: the one-node cavity kernel
             const unsigned grid = (unsigned)(((size_t)p.N + STEP_THREADS - 1) / STEP_THREADS);
             if (MODE != MODE_FIELDS && p.collision == 1) {
-                if constexpr (ST == ST_F32) cavity_kernel<ST, MHD, MODE, 1><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+                if constexpr (ST == ST_F32) e = launch_overlapped(cavity_kernel<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
             } else if (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS && p.variant == 0) {
                 if constexpr (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS) {
                     static const long long wave = resident_wave(cavity_kernel_coupled2<ST, MODE>, STEP_THREADS);
                     b.pf_ahead = (long long)grid > 4 * wave ? wave / 2 : 0;
-                    cavity_kernel_coupled2<ST, MODE><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+                    e = launch_overlapped(cavity_kernel_coupled2<ST, MODE>, grid, STEP_THREADS, st, p, b, fo);
                 }
             } else {
-                cavity_kernel<ST, MHD, MODE, 0><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+                e = launch_overlapped(cavity_kernel<ST, MHD, MODE, 0>, grid, STEP_THREADS, st, p, b, fo);
             }
             if (nblocks) *nblocks = grid;
-            return cudaGetLastError();
+            return e;
         }
     }
     if constexpr (MODE != MODE_FIELDS && (ST == ST_F32 || ST == ST_F32C || ST == ST_BF16)) {
         if (p.collision != 0) {   // preconditioned SRT-LBE: one node per thread
             const unsigned grid = (unsigned)(((size_t)p.N + STEP_THREADS - 1) / STEP_THREADS);
-            if (p.collision == 1) step_kernel_srt<ST, MHD, MODE, 1><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
-            else step_kernel_srt<ST, MHD, MODE, 2><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+            if (p.collision == 1) e = launch_overlapped(step_kernel_srt<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
+            else e = launch_overlapped(step_kernel_srt<ST, MHD, MODE, 2>, grid, STEP_THREADS, st, p, b, fo);
             if (nblocks) *nblocks = grid;
-            return cudaGetLastError();
+            return e;
         }
     }
     if constexpr (ST != ST_F32C && !Store<ST>::SR && MODE != MODE_FIELDS) {
@@ -2252,11 +2259,11 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
         if constexpr (!MHD && MODE != MODE_FIELDS && PMINB > 0) {
             static const long long wave = resident_wave(step_pair_kernel_dense<ST, MODE, PMINB>, PAIR_THREADS);
             b.pf_ahead = wave / 2;
-            step_pair_kernel_dense<ST, MODE, PMINB><<<grid, PAIR_THREADS, 0, st>>>(p, b);
+            e = launch_overlapped(step_pair_kernel_dense<ST, MODE, PMINB>, grid, PAIR_THREADS, st, p, b);
         } else {
             static const long long wave = resident_wave(step_pair_kernel<ST, MHD, MODE>, PAIR_THREADS);
             b.pf_ahead = wave / 2;
-            step_pair_kernel<ST, MHD, MODE><<<grid, PAIR_THREADS, 0, st>>>(p, b);
+            e = launch_overlapped(step_pair_kernel<ST, MHD, MODE>, grid, PAIR_THREADS, st, p, b);
         }
         if (nblocks) *nblocks = grid;
     } else {
@@ -2265,7 +2272,7 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
         if constexpr (!MHD && MODE == MODE_STEP && MINB > 0) {
             static const long long wave = resident_wave(step_kernel_dense<ST, MINB>, STEP_THREADS);
             b.pf_ahead = wave;
-            step_kernel_dense<ST, MINB><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+            e = launch_overlapped(step_kernel_dense<ST, MINB>, grid, STEP_THREADS, st, p, b, fo);
         } else if (MHD && (ST == ST_F32C || ((ST == ST_F32 || ST == ST_BF16) && MODE == MODE_STEP_RESID)) &&
                    MODE != MODE_FIELDS &&
                    p.variant == 0 && grid > 2 * one_pass_wave<ST, MODE>()) {
@@ -2284,16 +2291,16 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
                 // slower with it)
                 static const long long wave = resident_wave(step_kernel_coupled2<ST, MODE>, STEP_THREADS);
                 b.pf_ahead = ST != ST_BF16 && (long long)grid > 4 * wave ? wave / 2 : 0;
-                step_kernel_coupled2<ST, MODE><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+                e = launch_overlapped(step_kernel_coupled2<ST, MODE>, grid, STEP_THREADS, st, p, b, fo);
             }
         } else {
             static const long long wave = resident_wave(step_kernel<ST, MHD, MODE>, STEP_THREADS);
             b.pf_ahead = (MHD || MODE == MODE_STEP_RESID) ? wave / 2 : wave;
-            step_kernel<ST, MHD, MODE><<<grid, STEP_THREADS, 0, st>>>(p, b, fo);
+            e = launch_overlapped(step_kernel<ST, MHD, MODE>, grid, STEP_THREADS, st, p, b, fo);
         }
         if (nblocks) *nblocks = grid;
     }
-    return cudaGetLastError();
+    return e;
 }
 
 template <int ST>
