@@ -262,7 +262,9 @@ cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned thre
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // returned, so not left for the next check to find
+    return e;
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;"); }

@@ -192,7 +192,9 @@ cudaError_t resident_launch(K kernel, const ResidentPlan& pl, cudaStream_t st, c
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e != cudaSuccess) cudaGetLastError();   // returned, so not left for the next check to find
+    return e;
 }
 
 }  // namespace glbe

@@ -179,3 +179,32 @@ def test_two_streams_march_apart():
         _same(T.get_state(), out[k])
         T.close()
         S.close()
+
+
+@pytest.mark.parametrize("shape", [(4, 32, 4), (40, 40, 40), (80, 80, 72)])
+def test_captured_march_replays(shape):
+    """A march captured in the caller's graph (cluster, cooperative and overlapped launches) replays as the
+    same steps taken directly, its residual levels counted on the device."""
+    import torch
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        A = _solver(shape, "yz" if shape[2] > 4 else "y", "f32c", True)
+        _start(A)
+        A.step(20)
+        A.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            A.step(20)
+        for _ in range(3):
+            g.replay()
+        side.synchronize()
+        got = [x.clone() for x in A.get_state()]
+        levels = [h["t"] for h in A.history()]
+        A.sync()
+    B = _solver(shape, "yz" if shape[2] > 4 else "y", "f32c", True)
+    _start(B)
+    B.step(80)
+    _same(got, B.get_state())
+    assert levels == [h["t"] for h in B.history()] == [10, 20, 30, 40, 50, 60, 70]
+    A.close()
+    B.close()
