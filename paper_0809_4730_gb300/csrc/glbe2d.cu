@@ -66,18 +66,19 @@ static_assert(ex5(opp5(1)) == -1 && ey5(opp5(4)) == 1, "D2Q5 opposites");
 // Storage: FP32, BF16, or FP32 + FP16 remainder (compensated; the low parts
 // follow the high parts in the same buffer, scaled by 2^36).
 // ---------------------------------------------------------------------------
-// Read-only loads asking L2 for the whole 256-byte block (a warp reads 128
-// bytes of a population row, the next warp the following 128).
+// Loads asking L2 for the whole 256-byte block (a warp reads 128 bytes of a
+// population row, the next warp the following 128).  Coherent, as in the 3D
+// kernels: an overlapped launch begins while its predecessor writes these rows.
 __device__ __forceinline__ float ld256(const float* p)
 {
     float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ unsigned short ld256(const unsigned short* p)
 {
     unsigned short v;
-    asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
     return v;
 }
 
@@ -232,7 +233,7 @@ __device__ __forceinline__ void gather_f(const P2& p, const Nb& b, int x, int y,
         const int row = sol ? opp9t(a) : a;
         const int at = sol ? n : s;
         d[a] = S::ld(f + (size_t)row * p.N + at);
-        dl[a] = S::COMP ? __half2float(__ldg(fl + (size_t)row * p.N + at)) * LO2_INV : 0.f;
+        dl[a] = S::COMP ? __half2float(__ldca(fl + (size_t)row * p.N + at)) * LO2_INV : 0.f;
     }
 }
 
@@ -253,7 +254,7 @@ __device__ __forceinline__ void gather_g(const P2& p, const Nb& b, int x, int y,
         for (int j = 0; j < 2; ++j) {
             const int row = j * 5 + (sol ? opp5(a) : a);
             const float v = S::ld(g + (size_t)row * p.N + at);
-            const float vl = S::COMP ? __half2float(__ldg(gl + (size_t)row * p.N + at)) * LO2_INV : 0.f;
+            const float vl = S::COMP ? __half2float(__ldca(gl + (size_t)row * p.N + at)) * LO2_INV : 0.f;
             q[j * 5 + a] = sol ? -v : v;
             ql[j * 5 + a] = sol ? -vl : vl;
         }
@@ -273,7 +274,7 @@ __device__ __forceinline__ void gather_f_interior(const P2& p, int n, const void
     for (int a = 0; a < 9; ++a) {
         const ptrdiff_t k = (ptrdiff_t)a * p.N - (ex9(a) + ey9(a) * p.nx) + n;
         d[a] = S::ld(f + k);
-        dl[a] = S::COMP ? __half2float(__ldg(fl + k)) * LO2_INV : 0.f;
+        dl[a] = S::COMP ? __half2float(__ldca(fl + k)) * LO2_INV : 0.f;
     }
 }
 
@@ -289,7 +290,7 @@ __device__ __forceinline__ void gather_g_interior(const P2& p, int n, const void
         const int a = i % 5;
         const ptrdiff_t k = (ptrdiff_t)i * p.N - (ex5(a) + ey5(a) * p.nx) + n;
         q[i] = S::ld(g + k);
-        ql[i] = S::COMP ? __half2float(__ldg(gl + k)) * LO2_INV : 0.f;
+        ql[i] = S::COMP ? __half2float(__ldca(gl + k)) * LO2_INV : 0.f;
     }
 }
 
@@ -1198,7 +1199,7 @@ template <int ST> struct Pair2;
 template <> struct Pair2<GLBE_F32> {
     static __device__ __forceinline__ float2 ld(const void* base, size_t k)
     {
-        return __ldg(reinterpret_cast<const float2*>(static_cast<const float*>(base) + k));
+        return __ldca(reinterpret_cast<const float2*>(static_cast<const float*>(base) + k));
     }
     static __device__ __forceinline__ float ld1(const void* base, size_t k)
     {
@@ -1215,7 +1216,7 @@ template <> struct Pair2<GLBE_BF16> {
     static __device__ __forceinline__ float2 ld(const void* base, size_t k)
     {
         uint32_t u;
-        asm("ld.global.nc.L2::256B.b32 %0, [%1];"
+        asm volatile("ld.global.L2::256B.b32 %0, [%1];"
             : "=r"(u)
             : "l"(static_cast<const __nv_bfloat16*>(base) + k));
         return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));

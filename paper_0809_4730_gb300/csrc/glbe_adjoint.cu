@@ -94,9 +94,13 @@ __global__ void __launch_bounds__(ADJ_THREADS, 4) adjoint_kernel(const StepParam
     const size_t N = p.N;
     const bool inb = i < p.N;
     const uint32_t n = inb ? i : 0u;
-    const float* __restrict__ lf = a.lam_in;
-    const float* __restrict__ lg = a.lam_in + 19 * N;
-    const float* __restrict__ lk = a.lam_in + 40 * N;
+    // Not restrict: an overlapped launch begins while its predecessor still
+    // writes the cotangents (launch_overlapped), so they must not go through the
+    // read-only path.  (As asm volatile loads, which keep their order, they cost
+    // 3 us of 33 a coupled F32C sweep on 64^3.)
+    const float* lf = a.lam_in;
+    const float* lg = a.lam_in + 19 * N;
+    const float* lk = a.lam_in + 40 * N;
     float* __restrict__ of = a.lam_out;
     float* __restrict__ og = a.lam_out + 19 * N;
     float* __restrict__ ok = a.lam_out + 40 * N;
@@ -124,13 +128,13 @@ __global__ void __launch_bounds__(ADJ_THREADS, 4) adjoint_kernel(const StepParam
                 fold_lo(q, ql);
             }
         }
-        const float* __restrict__ l0 = lf + n;
+        const float* l0 = lf + n;
 #pragma unroll
         for (int o = 0; o < 19; ++o) vf[o] = *(seam_src(dir_opp(o), l0, l0 + wp, l0 + wm) + p.toff[o]);
         if (MHD) {
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const float* __restrict__ b0 = lg + (size_t)(j * 7) * N + n;
+                const float* b0 = lg + (size_t)(j * 7) * N + n;
 #pragma unroll
                 for (int o = 0; o < 7; ++o) vg[j * 7 + o] = *(seam_src(dir_opp(o), b0, b0 + wp, b0 + wm) + p.toff[o]);
             }
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 4) adjoint_kernel(const StepParam
             if (MHD) {
 #pragma unroll
                 for (int j = 0; j < 3; ++j) {
-                    const float* __restrict__ b = lg + (size_t)(j * 7) * N;
+                    const float* b = lg + (size_t)(j * 7) * N;
                     vg[j * 7] = b[n];
 #define GLBE_ADJG(a_, o_, src, sol) \
     vg[j * 7 + o_] = (sol) ? -b[(size_t)(a_) * N + n] : b[(size_t)(o_) * N + (src)];

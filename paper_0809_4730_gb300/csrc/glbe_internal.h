@@ -246,7 +246,8 @@ StepParams make_step_params(const glbe_params* p);
 // before it reads or writes anything, and the previous kernel, if it is one of
 // these, lets it begin once all its own blocks have started
 // (grid_dependency_release(); so no block waits for room that a waiting one
-// holds).  What is hidden is the launch and the first blocks' set-up, 2 to 4 us
+// holds).  What the previous kernel may still be writing then is read with
+// coherent loads only.  What is hidden is the launch and the first blocks' set-up, 2 to 4 us
 // a step: ten coupled F32 steps on 128^3 with fields 1297 -> 1263 us, twenty of
 // the 98^3 MHD cavity 2135 -> 2086 us, a 40-step transient's gradient on 64^3
 // 4298 -> 4083 us.

@@ -144,43 +144,46 @@ constexpr float LO_SCALE = 68719476736.0f;        // 2^36
 constexpr float LO_INV = 1.4551915228366852e-11f; // 2^-36
 
 template <int ST> struct Store;
-// Read-only load asking L2 for the whole 256-byte block: a warp reads 128
+// Load asking L2 for the whole 256-byte block: a warp reads 128
 // bytes of a population row and the next warp the following 128 (measured:
 // F32 step 0.888 against 0.893 ms, F16 paired step 0.509 against 0.517 ms,
 // BF16 paired step 0.485 against 0.489 ms, steady adjoint iteration 0.2455
-// against 0.2462 ms)
-__device__ __forceinline__ float ldg_l2_256(const float* p)
+// against 0.2462 ms).  Coherent, like every load here of what an earlier step
+// wrote: an overlapped launch (launch_overlapped) begins while its
+// predecessor still writes these rows, and the non-coherent path (ld.global.nc,
+// __ldg) is only for data that nobody writes while the kernel lives.
+__device__ __forceinline__ float ld_l2_256(const float* p)
 {
     float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint32_t ldg_l2_256(const uint32_t* p)
+__device__ __forceinline__ uint32_t ld_l2_256(const uint32_t* p)
 {
     uint32_t v;
-    asm("ld.global.nc.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 
 template <> struct Store<ST_F32> {
     using T = float;
     static constexpr bool COMP = false, SCALED = false, SR = false;
-    static __device__ __forceinline__ float ld(const T* p) { return ldg_l2_256(p); }
+    static __device__ __forceinline__ float ld(const T* p) { return ld_l2_256(p); }
     static __device__ __forceinline__ T cv(float v) { return v; }
-    static __device__ __forceinline__ F2 ld2(const T* p) { return F2(__ldg(reinterpret_cast<const float2*>(p))); }
+    static __device__ __forceinline__ F2 ld2(const T* p) { return F2(__ldca(reinterpret_cast<const float2*>(p))); }
     static __device__ __forceinline__ void st2(T* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
 };
 template <> struct Store<ST_BF16> {
     using T = __nv_bfloat16;
     static constexpr bool COMP = false, SCALED = false, SR = false;
-    static __device__ __forceinline__ float ld(const T* p) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ float ld(const T* p) { return __bfloat162float(__ldca(p)); }
     static __device__ __forceinline__ T cv(float v) { return __float2bfloat16_rn(v); }
     // a BF16 value is the high half of the FP32 with the same bits: the pair
     // is widened from one 32-bit load by a shift and a mask (exact; measured
     // 0.584 against 0.620 ms per paired step with __bfloat1622float2)
     static __device__ __forceinline__ F2 ld2(const T* p)
     {
-        const uint32_t u = ldg_l2_256(reinterpret_cast<const uint32_t*>(p));
+        const uint32_t u = ld_l2_256(reinterpret_cast<const uint32_t*>(p));
         return F2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
     }
     static __device__ __forceinline__ void st2(T* p, F2 v)
@@ -191,11 +194,11 @@ template <> struct Store<ST_BF16> {
 template <> struct Store<ST_F16> {
     using T = __half;
     static constexpr bool COMP = false, SCALED = true, SR = false;
-    static __device__ __forceinline__ float ld(const T* p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float ld(const T* p) { return __half2float(__ldca(p)); }
     static __device__ __forceinline__ T cv(float v) { return __float2half_rn(v); }
     static __device__ __forceinline__ F2 ld2(const T* p)
     {
-        const uint32_t u = ldg_l2_256(reinterpret_cast<const uint32_t*>(p));
+        const uint32_t u = ld_l2_256(reinterpret_cast<const uint32_t*>(p));
         __half2 h;
         memcpy(&h, &u, 4);
         return F2(__half22float2(h));
@@ -205,15 +208,15 @@ template <> struct Store<ST_F16> {
 template <> struct Store<ST_F32C> {
     using T = float;
     static constexpr bool COMP = true, SCALED = false, SR = false;
-    static __device__ __forceinline__ float ld(const T* p) { return ldg_l2_256(p); }
+    static __device__ __forceinline__ float ld(const T* p) { return ld_l2_256(p); }
     static __device__ __forceinline__ T cv(float v) { return v; }
-    static __device__ __forceinline__ F2 ld2(const T* p) { return F2(__ldg(reinterpret_cast<const float2*>(p))); }
+    static __device__ __forceinline__ F2 ld2(const T* p) { return F2(__ldca(reinterpret_cast<const float2*>(p))); }
     static __device__ __forceinline__ void st2(T* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
-    static __device__ __forceinline__ float ld_lo(const __half* p) { return __half2float(__ldg(p)) * LO_INV; }
+    static __device__ __forceinline__ float ld_lo(const __half* p) { return __half2float(__ldca(p)) * LO_INV; }
     static __device__ __forceinline__ __half cv_lo(float v) { return __float2half_rn(v * LO_SCALE); }
     static __device__ __forceinline__ F2 ld2_lo(const __half* p)
     {
-        const float2 w = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+        const float2 w = __half22float2(__ldca(reinterpret_cast<const __half2*>(p)));
         return F2(w.x * LO_INV, w.y * LO_INV);
     }
     static __device__ __forceinline__ void st2_lo(__half* p, F2 v)
@@ -295,7 +298,7 @@ struct SrBits {
 template <int ST>
 __device__ __forceinline__ uint32_t step_seed(const StepBuffers& b)
 {
-    if constexpr (Store<ST>::SR) return b.sr_ctr ? __ldg(b.sr_ctr + b.sr_par) : b.sr_seed;
+    if constexpr (Store<ST>::SR) return b.sr_ctr ? __ldca(b.sr_ctr + b.sr_par) : b.sr_seed;
     else return 0u;
 }
 // One thread of the step writes the next step's seed; no block of this step
@@ -328,8 +331,8 @@ __device__ __forceinline__ void store_pair(typename Store<ST>::T* p, F1 v, SrBit
 }
 
 // Loads of populations written earlier in the same launch (the persistent
-// batch kernel) must not use the non-coherent read-only path.  CG = true
-// gathers with coherent loads that are still cached in L1 (ld.global.ca):
+// batch kernel, the resident marches): CG = true gathers with loads that are
+// still cached in L1 (ld.global.ca), without the request for the L2 block:
 // the gpu-scope fences of the grid barrier between levels order them after
 // the previous level's stores, and no buffer is written in the level that
 // reads it.  The second gather of a coupled node's two-pass update then hits
