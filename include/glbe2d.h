@@ -113,6 +113,9 @@ glbe_status glbe2d_set_force(glbe2d_ctx* ctx, const float* d_F);
  * about 600,000 nodes) take n >= 2 steps in one launch, as in glbe_step_n. */
 glbe_status glbe2d_step_n(glbe2d_ctx* ctx, long n);
 
+/* As glbe_set_barrier_test. */
+glbe_status glbe2d_set_barrier_test(glbe2d_ctx* ctx, long long spin_limit, int absent_block);
+
 /* Synchronises and returns the latest residual record (momentum[2] = 0).
  * GLBE_ERR_DIVERGED if it saw a non-finite velocity. */
 glbe_status glbe2d_residual(glbe2d_ctx* ctx, glbe_residual_info* out);

@@ -1041,6 +1041,7 @@ __global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, M
     __shared__ int verdict;
     const int BT = blockDim.x, G = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = BT >> 5;
     if (m.solve && *(volatile int*)m.out.stop) return;   // converged in an earlier launch
+    if (!CLUSTER && (int)blockIdx.x == m.absent) return;
     const uint32_t ntiles = ((uint32_t)p.N + BT - 1) / BT;
     int mine = 0;
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, ++mine)
@@ -1126,7 +1127,7 @@ __global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, M
             }
         } else {
             if (sums && threadIdx.x < RES_SUMS) m.partials[(size_t)threadIdx.x * G + blockIdx.x] = bsum[threadIdx.x];
-            if (!resident_barrier(m.bar, gen)) return;
+            if (!resident_barrier(m.bar, gen, m.spin_limit)) return;
             if (sums && (m.solve || writer)) {
                 // a solve's blocks all take the decision (num, den, non-finite count), from the same numbers in
                 // the same order
@@ -1488,8 +1489,11 @@ __global__ void __launch_bounds__(T2D) set_state2d_kernel(const P2 p, void* fsrc
 }
 
 __global__ void ctl2d_kernel(long long* t_dev, long long t, int* stop, int stop_v, double* tol, double tol_v,
-                             double* record, unsigned long long* hist_count, int reset_record)
+                             double* record, unsigned long long* hist_count, int reset_record,
+                             unsigned* bar = nullptr)
 {
+    if (bar)
+        for (int k = 0; k < RES_BAR_WORDS; ++k) bar[k] = 0u;
     if (t_dev) *t_dev = t;
     if (stop) *stop = stop_v;
     if (tol) *tol = tol_v;
@@ -1657,6 +1661,8 @@ struct glbe2d_ctx {
     cudaGraphExec_t chunk;
     unsigned* res_bar;      // barrier words of the resident march (count, generation, error)
     ResidentPlan res;       // form 0: steps are launched one by one
+    unsigned res_spin;      // polls of a barrier wait before it gives up
+    int res_absent;         // block that leaves a march at once (failure test), or -1
     bool res_used;          // a resident march was launched since the error flag was last read
 };
 
@@ -1844,6 +1850,8 @@ glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
     m.tol = tol;
     m.out = RecordOut{c->record, c->hist, c->hist_count, HIST_CAP2, c->t_dev, c->stop_dev, c->tol_dev, c->mass0};
     m.bar = c->res_bar;
+    m.spin_limit = c->res_spin;
+    m.absent = c->res_absent;
     const bool mhd = c->prm.induction;
     cudaError_t e;
     switch (c->prm.storage) {
@@ -1874,7 +1882,6 @@ glbe_status sync_control2(glbe2d_ctx* c, int* stop)
     unsigned err = 0;
     std::memcpy(&err, misc + (reinterpret_cast<char*>(c->res_bar + 2) - base), sizeof err);
     if (!err) return GLBE_OK;
-    GLBE2D_CUDA(cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream), "2D resident march reset");
     return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
 }
 
@@ -2002,6 +2009,8 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->stop_dev = reinterpret_cast<int*>(misc + 24);
     c->res_bar = reinterpret_cast<unsigned*>(misc + 32);
     c->res = plan_resident2(c);
+    c->res_spin = RES_SPIN_LIMIT;
+    c->res_absent = -1;
     c->res_used = false;
     c->mass0 = p->rho0 * (double)fluid2(p);
     c->t = 0;
@@ -2009,9 +2018,9 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->stream = static_cast<cudaStream_t>(p->stream);
     // the rest state: every deviation, the Lorentz force and the field zero
     cudaError_t e = cudaMemsetAsync(d_workspace, 0, L.record, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess) {
-        ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record, c->hist_count, 1);
+        ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record, c->hist_count, 1,
+                                             c->res_bar);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -2204,7 +2213,7 @@ glbe_status glbe2d_set_state(glbe2d_ctx* c, const float* d_df, const float* d_dg
     }
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state kernel");
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, ((long long)t + 9) / 10 * 10, c->stop_dev, 0, c->tol_dev, 0.0,
-                                         c->record, c->hist_count, 1);
+                                         c->record, c->hist_count, 1, c->res_bar);
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state reset");
     return GLBE_OK;
 }
@@ -2222,6 +2231,16 @@ glbe_status glbe2d_sync(glbe2d_ctx* c)
     const glbe_status s = sync_control2(c, nullptr);
     if (s != GLBE_OK) return s;
     GLBE2D_CUDA(cudaGetLastError(), "2D async error");
+    return GLBE_OK;
+}
+
+glbe_status glbe2d_set_barrier_test(glbe2d_ctx* c, long long spin_limit, int absent_block)
+{
+    if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
+    if (spin_limit < 1 || spin_limit > 0x7fffffffll) return fail(GLBE_ERR_ARG, "spin_limit must be in [1, 2^31)");
+    if (c->res.form < 2) return fail(GLBE_ERR_STATE, "this context's steps do not meet at a counting barrier");
+    c->res_spin = (unsigned)spin_limit;
+    c->res_absent = absent_block < 0 ? -1 : absent_block;
     return GLBE_OK;
 }
 

@@ -322,8 +322,11 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(double* __restric
 }
 
 __global__ void misc_set_kernel(long long* t_dev, long long t, int* stop, int stop_v, double* tol, double tol_v,
-                                double* record, unsigned long long* hist_count, int reset_record)
+                                double* record, unsigned long long* hist_count, int reset_record,
+                                unsigned* bar = nullptr)
 {
+    if (bar)
+        for (int k = 0; k < RES_BAR_WORDS; ++k) bar[k] = 0u;
     if (t_dev) *t_dev = t;
     if (stop) *stop = stop_v;
     if (tol) *tol = tol_v;
@@ -357,6 +360,8 @@ struct glbe_ctx {
     double* tol_dev;
     unsigned* res_bar;       // barrier words of the resident march (count, generation, error)
     ResidentPlan res;        // form 0: steps are launched one by one
+    unsigned res_spin;       // polls of a barrier wait before it gives up
+    int res_absent;          // block that leaves a march at once (failure test), or -1
     bool res_used;           // a resident march was launched since the error flag was last read
     unsigned* sr_ctr;   // [2] seeds of stochastic rounding, read by the step of parity t & 1
     double mass0;   // rho0 x number of fluid nodes
@@ -455,6 +460,8 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
     m.tol = tol;
     m.out = RecordOut{c->record, c->hist, c->hist_count, HIST_CAP, c->t_dev, c->stop_dev, c->tol_dev, c->mass0};
     m.bar = c->res_bar;
+    m.spin_limit = c->res_spin;
+    m.absent = c->res_absent;
     const bool mhd = c->prm.induction;
     cudaError_t e;
     switch (c->prm.storage) {
@@ -487,7 +494,6 @@ glbe_status sync_control(glbe_ctx* c, int* stop)
     unsigned err = 0;
     std::memcpy(&err, misc + ((const char*)(c->res_bar + 2) - (c->ws + c->L.misc)), sizeof err);
     if (!err) return GLBE_OK;
-    GLBE_CUDA(cudaMemsetAsync(c->res_bar, 0, 3 * sizeof(unsigned), c->stream), "resident march reset");
     return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
 }
 
@@ -632,6 +638,8 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     c->sr_ctr = reinterpret_cast<unsigned*>(misc + 32);
     c->res_bar = reinterpret_cast<unsigned*>(misc + 40);
     c->res = plan_resident(c);
+    c->res_spin = RES_SPIN_LIMIT;
+    c->res_absent = -1;
     c->res_used = false;
     c->mass0 = p->rho0 * (double)fluid_nodes(p);   // planes on walls and ghost planes excluded
     c->t = 0;
@@ -647,7 +655,7 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->ws + L.usnap, 0, snap_rows(p->storage) * c->N * sizeof(float), c->stream);
     // the seeds and the barrier words behind them
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->sr_ctr, 0, 5 * sizeof(unsigned), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->sr_ctr, 0, (2 + RES_BAR_WORDS) * sizeof(unsigned), c->stream);
     if (e == cudaSuccess && c->sp.cavity) {   // the lid's links of the first gather (see lid_init_kernel)
         if (p->storage == GLBE_F32) e = launch_lid_init_t<ST_F32>(c->sp, c->f[0], c->stream);
         else if (p->storage == GLBE_F32C) e = launch_lid_init_t<ST_F32C>(c->sp, c->f[0], c->stream);
@@ -760,6 +768,16 @@ glbe_status glbe_sync(glbe_ctx* c)
     }
     if (waited_out) return fail(GLBE_ERR_TIMEOUT, "a pipeline wait of the TMA-staged step kernel ran out");
     return sync_control(c, nullptr);
+}
+
+glbe_status glbe_set_barrier_test(glbe_ctx* c, long long spin_limit, int absent_block)
+{
+    if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
+    if (spin_limit < 1 || spin_limit > 0x7fffffffll) return fail(GLBE_ERR_ARG, "spin_limit must be in [1, 2^31)");
+    if (c->res.form < 2) return fail(GLBE_ERR_STATE, "this context's steps do not meet at a counting barrier");
+    c->res_spin = (unsigned)spin_limit;
+    c->res_absent = absent_block < 0 ? -1 : absent_block;
+    return GLBE_OK;
 }
 
 static glbe_status read_record(glbe_ctx* c, glbe_residual_info* out)
@@ -966,7 +984,7 @@ glbe_status glbe_set_state(glbe_ctx* c, const float* d_df, const float* d_dg, co
     GLBE_CUDA(e, "set_state kernel");
     // a replaced state starts a fresh residual history
     misc_set_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, (long long)t + 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record,
-                                            c->hist_count, 1);
+                                            c->hist_count, 1, c->res_bar);
     GLBE_CUDA(cudaGetLastError(), "set_state reset");
     c->t = t;
     c->t_snap = -1;
@@ -1097,7 +1115,7 @@ extern "C" glbe_status glbe_checkpoint_load(glbe_ctx* c, const void* h_buf, size
     GLBE_CUDA(cudaMemcpy(c->record, in, RECORD_STRIDE * sizeof(double), cudaMemcpyHostToDevice), "restore record");
     // residual level counter as saved; a fresh history; no pending stop
     misc_set_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, (long long)h.t_dev, c->stop_dev, 0, c->tol_dev, 0.0, nullptr,
-                                            nullptr, 0);
+                                            nullptr, 0, c->res_bar);
     GLBE_CUDA(cudaGetLastError(), "restore counters");
     GLBE_CUDA(cudaMemsetAsync(c->hist_count, 0, sizeof(unsigned long long), c->stream), "restore history");
     const unsigned seed = (unsigned)h.reserved[0];

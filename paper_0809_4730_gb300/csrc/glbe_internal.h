@@ -199,8 +199,15 @@ struct ResidentMarch {
     int solve;
     double tol;
     RecordOut out;
-    unsigned* bar;        // barrier count, barrier generation, error flag
+    // Barrier count, barrier generation, and a flag that a wait ran out: the
+    // state is then incomplete and the count stale, so every march ends at its
+    // first barrier until the three words are zero again (with a new state).
+    unsigned* bar;
+    unsigned spin_limit;  // polls of a barrier wait before it gives up (looked at every 4096)
+    int absent;           // block that leaves the launch at once (failure test), or -1
 };
+constexpr int RES_BAR_WORDS = 3;
+constexpr unsigned RES_SPIN_LIMIT = 1u << 24;   // several seconds
 
 constexpr long RES_MOST_STEPS = 1000000;   // steps of one launch
 

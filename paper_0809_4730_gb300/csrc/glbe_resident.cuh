@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
     __shared__ int verdict;
     const int BT = blockDim.x, G = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (m.solve && *(volatile int*)m.out.stop) return;   // converged in an earlier launch
+    if (!CLUSTER && (int)blockIdx.x == m.absent) return;
     const uint32_t units = UNIT == RES_PAIR ? p.N >> 1 : p.N, ntiles = (units + BT - 1) / BT;
     int mine = 0;
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, ++mine) {
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
             }
         }
         if constexpr (CLUSTER) cluster_level_barrier();
-        else if (!resident_barrier(m.bar, gen)) return;
+        else if (!resident_barrier(m.bar, gen, m.spin_limit)) return;
         if (resid) {
             if (snap && (m.solve || writer)) {
                 // a solve's blocks all take the decision, from the same sums in the same order

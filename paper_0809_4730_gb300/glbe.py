@@ -108,6 +108,8 @@ _SIGNATURES = {
     "glbe_batch_destroy": (None, [C.c_void_p]),
     "glbe_step_residual_noalloc": (C.c_int, [_P(glbe_params), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                              C.c_int, C.c_long, _P(glbe_residual_info)]),
+    "glbe_set_barrier_test": (C.c_int, [C.c_void_p, C.c_longlong, C.c_int]),
+    "glbe2d_set_barrier_test": (C.c_int, [C.c_void_p, C.c_longlong, C.c_int]),
     "glbe_halo_bytes": (C.c_int, [C.c_void_p, _P(C.c_size_t)]),
     "glbe_halo_pack": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
     "glbe_halo_unpack": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
@@ -509,6 +511,9 @@ class Solver2D:
         glbe2d_set_state(self.ctx, df.contiguous(), None if dg is None else dg.contiguous(),
                          None if FL is None else FL.contiguous(), t)
 
+    def set_barrier_test(self, spin_limit: int, absent_block: int):
+        _check(load().glbe2d_set_barrier_test(self.ctx, int(spin_limit), int(absent_block)), "glbe2d_set_barrier_test")
+
     def sync(self):
         glbe2d_sync(self.ctx)
 
@@ -707,6 +712,9 @@ class Solver:
     def set_state(self, df, dg=None, FL=None, t: int = 0):
         glbe_set_state(self.ctx, df.contiguous(), None if dg is None else dg.contiguous(),
                        None if FL is None else FL.contiguous(), t)
+
+    def set_barrier_test(self, spin_limit: int, absent_block: int):
+        _check(load().glbe_set_barrier_test(self.ctx, int(spin_limit), int(absent_block)), "glbe_set_barrier_test")
 
     def sync(self):
         glbe_sync(self.ctx)

@@ -1,0 +1,96 @@
+"""A barrier wait of a resident march that runs out: one block leaves the launch at once, so the others' first
+wait ends at a short poll limit.  The march must not hang, the host must learn of it, nothing may march from
+the incomplete state, and a new state must march as in a context that never failed."""
+import pytest
+
+from test_gpu_resident import _same, _solver, _start
+
+pytestmark = pytest.mark.gpu
+
+LIMIT = 1 << 14          # polls: some ten milliseconds
+# one tile a block and several tiles a block, in pairs and one node a thread
+CASES = [((32, 32, 9), "f32", True), ((48, 48, 48), "f32", False), ((48, 48, 48), "f32c", True),
+         ((51, 48, 48), "bf16", False)]
+
+
+def _status(call):
+    from paper_0809_4730_gb300.glbe import GlbeError
+    with pytest.raises(GlbeError) as e:
+        call()
+    return e.value.status
+
+
+def _timed_out(S, absent=0):
+    S.set_barrier_test(LIMIT, absent)
+    S.step(13)
+    S.set_barrier_test(1 << 24, -1)
+
+
+def _solver2(mhd, storage, shape=(128, 304)):
+    from paper_0809_4730_gb300.glbe import Solver2D
+    kw = dict(wall_lo=(0, 1), wall_hi=(0, 1), gamma=0.2, nu=0.05, F=(2e-6, 1e-6), storage=storage)
+    if mhd:
+        kw.update(induction=1, gamma_m=0.2, eta=0.05, chi=0.05, mu=1.0, B0=(0.002, 0.004))
+    return Solver2D(*shape, **kw)
+
+
+def _state2(S):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda q, s: s * (2 * torch.rand(q, S.N, device="cuda", generator=g) - 1)  # noqa: E731
+    S.set_state(r(9, 1e-4), r(10, 1e-5) if S.induction else None, r(2, 1e-7) if S.induction else None, 0)
+
+
+@pytest.mark.parametrize("reported", [True, False])
+@pytest.mark.parametrize("shape,storage,mhd", CASES)
+def test_a_new_state_marches_as_before(shape, storage, mhd, reported):
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
+    A, B = _solver(shape, "y", storage, mhd), _solver(shape, "y", storage, mhd)
+    _start(B)
+    data = B.checkpoint()
+    for _ in range(23):
+        B.step(1)
+    for restore in (lambda: _start(A), lambda: A.restore(data)):
+        _start(A)
+        A.step(4)
+        _timed_out(A)
+        A.step(20)                            # does not march: the barrier's count is stale
+        if reported:
+            assert _status(A.sync) == GLBE_ERR_TIMEOUT
+        restore()
+        A.step(23)
+        A.sync()
+        _same(A.get_state(), B.get_state())
+        assert [h["t"] for h in A.history()] == [10, 20]
+    A.close()
+    B.close()
+
+
+@pytest.mark.parametrize("storage,mhd", [("f32", False), ("f32c", True)])
+def test_2d_a_new_state_marches_as_before(storage, mhd):
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
+    A, B = _solver2(mhd, storage), _solver2(mhd, storage)
+    _state2(B)
+    for _ in range(23):
+        B.step(1)
+    _state2(A)
+    A.step(4)
+    _timed_out(A, absent=1)
+    A.step(20)
+    assert _status(A.sync) == GLBE_ERR_TIMEOUT
+    _state2(A)
+    A.step(23)
+    A.sync()
+    _same(A.get_state(), B.get_state())
+    A.close()
+    B.close()
+
+
+def test_contexts_without_a_counting_barrier_refuse_the_hook():
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_ARG, GLBE_ERR_STATE
+    for S in (_solver((4, 32, 4), "y", "f32", False), _solver((48, 48, 48), "y", "f32", False, variant=1)):
+        assert _status(lambda: S.set_barrier_test(LIMIT, 0)) == GLBE_ERR_STATE
+        S.close()
+    S = _solver((48, 48, 48), "y", "f32", False)
+    assert _status(lambda: S.set_barrier_test(0, 0)) == GLBE_ERR_ARG
+    S.close()
