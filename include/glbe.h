@@ -196,14 +196,17 @@ glbe_status glbe_set_force_host(glbe_ctx* ctx, const float* h_F);
  * the automatic kernel form, small grids (up to about 350,000 nodes) take
  * n >= 2 steps in one launch whose blocks stay resident and meet at a bounded
  * barrier between levels: the same states bit for bit.  Should a wait run out,
- * the state is incomplete: the next call that synchronises returns
- * GLBE_ERR_TIMEOUT, and no such launch marches again until glbe_set_state or
- * glbe_checkpoint_load gives the context a state. */
+ * the state is incomplete: no such launch marches again and every call that
+ * synchronises (glbe_sync, glbe_residual, glbe_history, glbe_checkpoint_save,
+ * glbe_solve) returns GLBE_ERR_TIMEOUT, the adjoint calls, once it is known,
+ * GLBE_ERR_STATE, until glbe_set_state or glbe_checkpoint_load gives the context
+ * a state. */
 glbe_status glbe_step_n(glbe_ctx* ctx, long n);
 
 /* Failure detection of those launches: a barrier wait gives up after
- * spin_limit polls (looked at every 4096; default 2^24, several seconds); absent_block >= 0 makes
- * that block leave every such launch at once (for tests), -1 none.
+ * spin_limit polls (looked at every 4096; default 2^24, several seconds);
+ * absent_block >= 0 makes that block leave every such launch at once (for
+ * tests), -1 none.
  * GLBE_ERR_STATE where the context's steps meet at no such barrier (launched
  * one by one, or one thread-block cluster). */
 glbe_status glbe_set_barrier_test(glbe_ctx* ctx, long long spin_limit, int absent_block);

@@ -1664,6 +1664,7 @@ struct glbe2d_ctx {
     unsigned res_spin;      // polls of a barrier wait before it gives up
     int res_absent;         // block that leaves a march at once (failure test), or -1
     bool res_used;          // a resident march was launched since the error flag was last read
+    bool torn;              // a barrier wait ran out and no state was set since
 };
 
 namespace {
@@ -1867,7 +1868,8 @@ glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
 }
 
 // Waits for the stream and reports whether a barrier wait of a resident march
-// ran out; stop (may be NULL) receives the march's stop flag.
+// ran out, from then on until a state is set; stop (may be NULL) receives the
+// march's stop flag.
 glbe_status sync_control2(glbe2d_ctx* c, int* stop)
 {
     const bool resident = c->res_used && c->res.form >= 2;
@@ -1878,11 +1880,11 @@ glbe_status sync_control2(glbe2d_ctx* c, int* stop)
         GLBE2D_CUDA(cudaMemcpyAsync(misc, base, sizeof misc, cudaMemcpyDeviceToHost, c->stream), "2D control words");
     GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D sync");
     if (stop) std::memcpy(stop, misc + (reinterpret_cast<char*>(c->stop_dev) - base), sizeof *stop);
-    if (!resident) return GLBE_OK;
     unsigned err = 0;
-    std::memcpy(&err, misc + (reinterpret_cast<char*>(c->res_bar + 2) - base), sizeof err);
-    if (!err) return GLBE_OK;
-    return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
+    if (resident) std::memcpy(&err, misc + (reinterpret_cast<char*>(c->res_bar + 2) - base), sizeof err);
+    if (err) c->torn = true;
+    if (c->torn) return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out: the state is incomplete");
+    return GLBE_OK;
 }
 
 glbe_status read_record2(glbe2d_ctx* c, glbe_residual_info* out)
@@ -2012,6 +2014,7 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
+    c->torn = false;
     c->mass0 = p->rho0 * (double)fluid2(p);
     c->t = 0;
     c->t_snap = -1;
@@ -2070,7 +2073,8 @@ glbe_status glbe2d_history(glbe2d_ctx* c, glbe_residual_info* out, long cap, lon
     *n = 0;
     if (cap <= 0) return GLBE_OK;
     unsigned long long count = 0;
-    GLBE2D_CUDA(cudaStreamSynchronize(c->stream), "2D history sync");
+    const glbe_status s = sync_control2(c, nullptr);
+    if (s != GLBE_OK) return s;
     GLBE2D_CUDA(cudaMemcpy(&count, c->hist_count, sizeof count, cudaMemcpyDeviceToHost), "2D history count");
     const unsigned long long kept = count < HIST_CAP2 ? count : HIST_CAP2;
     const unsigned long long take = kept < (unsigned long long)cap ? kept : (unsigned long long)cap;
@@ -2215,6 +2219,7 @@ glbe_status glbe2d_set_state(glbe2d_ctx* c, const float* d_df, const float* d_dg
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, ((long long)t + 9) / 10 * 10, c->stop_dev, 0, c->tol_dev, 0.0,
                                          c->record, c->hist_count, 1, c->res_bar);
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state reset");
+    c->torn = false;
     return GLBE_OK;
 }
 

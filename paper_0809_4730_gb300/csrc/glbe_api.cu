@@ -363,6 +363,7 @@ struct glbe_ctx {
     unsigned res_spin;       // polls of a barrier wait before it gives up
     int res_absent;          // block that leaves a march at once (failure test), or -1
     bool res_used;           // a resident march was launched since the error flag was last read
+    bool torn;               // a barrier wait ran out and no state was set since
     unsigned* sr_ctr;   // [2] seeds of stochastic rounding, read by the step of parity t & 1
     double mass0;   // rho0 x number of fluid nodes
     long t;         // current time level
@@ -478,8 +479,9 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
 }
 
 // Waits for the stream and reports whether a barrier wait of a resident march
-// ran out; stop (may be NULL) receives the march's stop flag.  One copy of the
-// control words, on the context's own stream.
+// ran out, from then on until a state is set; stop (may be NULL) receives the
+// march's stop flag.  One copy of the control words, on the context's own
+// stream.  Every call that synchronises does it here.
 glbe_status sync_control(glbe_ctx* c, int* stop)
 {
     const bool resident = c->res_used && c->res.form >= 2;
@@ -490,11 +492,11 @@ glbe_status sync_control(glbe_ctx* c, int* stop)
                   "control words");
     GLBE_CUDA(cudaStreamSynchronize(c->stream), "sync");
     if (stop) std::memcpy(stop, misc + ((const char*)c->stop_dev - (c->ws + c->L.misc)), sizeof *stop);
-    if (!resident) return GLBE_OK;
     unsigned err = 0;
-    std::memcpy(&err, misc + ((const char*)(c->res_bar + 2) - (c->ws + c->L.misc)), sizeof err);
-    if (!err) return GLBE_OK;
-    return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out");
+    if (resident) std::memcpy(&err, misc + ((const char*)(c->res_bar + 2) - (c->ws + c->L.misc)), sizeof err);
+    if (err) c->torn = true;
+    if (c->torn) return fail(GLBE_ERR_TIMEOUT, "a barrier wait of the resident march ran out: the state is incomplete");
+    return GLBE_OK;
 }
 
 // Enqueues the step from level c->t to c->t + 1 on stream st.
@@ -532,6 +534,7 @@ size_t storage_value_bytes(int storage) { return storage_bytes(storage); }
 glbe_status ctx_view(glbe_ctx* c, CtxView* v)
 {
     if (!c || !v) return fail(GLBE_ERR_ARG, "ctx or view is NULL");
+    if (c->torn) return fail(GLBE_ERR_STATE, "the state is incomplete: a barrier wait of the resident march ran out");
     const int s = (int)(c->t & 1);
     v->prm = c->prm;
     v->sp = c->sp;
@@ -546,6 +549,8 @@ glbe_status ctx_view(glbe_ctx* c, CtxView* v)
     v->stream = c->stream;
     return GLBE_OK;
 }
+
+glbe_status ctx_sync(glbe_ctx* c) { return sync_control(c, nullptr); }
 
 cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, long long* t_dev, double* record,
                             double* hist, unsigned long long* hist_count, unsigned hist_cap, int* stop,
@@ -641,6 +646,7 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
+    c->torn = false;
     c->mass0 = p->rho0 * (double)fluid_nodes(p);   // planes on walls and ghost planes excluded
     c->t = 0;
     c->t_snap = -1;
@@ -806,7 +812,8 @@ glbe_status glbe_history(glbe_ctx* c, glbe_residual_info* out, long cap, long* n
     *n = 0;
     if (cap <= 0) return GLBE_OK;
     unsigned long long count = 0;
-    GLBE_CUDA(cudaStreamSynchronize(c->stream), "history sync");
+    const glbe_status s = sync_control(c, nullptr);
+    if (s != GLBE_OK) return s;
     GLBE_CUDA(cudaMemcpy(&count, c->hist_count, sizeof count, cudaMemcpyDeviceToHost), "history count");
     const unsigned long long kept = count < HIST_CAP ? count : HIST_CAP;
     const unsigned long long take = kept < (unsigned long long)cap ? kept : (unsigned long long)cap;
@@ -986,6 +993,7 @@ glbe_status glbe_set_state(glbe_ctx* c, const float* d_df, const float* d_dg, co
     misc_set_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, (long long)t + 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record,
                                             c->hist_count, 1, c->res_bar);
     GLBE_CUDA(cudaGetLastError(), "set_state reset");
+    c->torn = false;
     c->t = t;
     c->t_snap = -1;
     return GLBE_OK;
@@ -1033,7 +1041,8 @@ extern "C" glbe_status glbe_checkpoint_save(glbe_ctx* c, void* h_buf, size_t byt
     if (!c || !h_buf) return fail(GLBE_ERR_ARG, "ctx or buffer is NULL");
     const size_t total = ckpt_total(c);
     if (bytes < total) return fail(GLBE_ERR_ARG, "checkpoint buffer of %zu bytes is smaller than %zu", bytes, total);
-    GLBE_CUDA(cudaStreamSynchronize(c->stream), "checkpoint sync");
+    const glbe_status st = sync_control(c, nullptr);
+    if (st != GLBE_OK) return st;
     CkptHeader h{};
     std::memcpy(h.magic, "GLBECKP1", 8);
     h.version = 1;
@@ -1122,6 +1131,7 @@ extern "C" glbe_status glbe_checkpoint_load(glbe_ctx* c, const void* h_buf, size
     GLBE_CUDA(cudaMemcpyAsync(c->sr_ctr + (h.t & 1), &seed, sizeof seed, cudaMemcpyHostToDevice, c->stream),
               "restore seed");
     GLBE_CUDA(cudaStreamSynchronize(c->stream), "restore sync");
+    c->torn = c->res_used = false;   // the words are zero and nothing is in flight
     c->t = (long)h.t;
     c->t_snap = (long)h.t_snap;
     return GLBE_OK;

@@ -295,7 +295,10 @@ struct CtxView {
     size_t g_bytes;       // bytes of one g buffer (0 without induction)
     cudaStream_t stream;
 };
-glbe_status ctx_view(glbe_ctx* c, CtxView* v);
+glbe_status ctx_view(glbe_ctx* c, CtxView* v);   // GLBE_ERR_STATE when the state is known to be incomplete
+// Waits for the context's stream; GLBE_ERR_TIMEOUT when a barrier wait of a
+// resident march ran out and no state was set since.
+glbe_status ctx_sync(glbe_ctx* c);
 
 // NVTX range around a C-ABI call (visible in Nsight tools; header-only NVTX 3,
 // a no-op unless a tool is attached).

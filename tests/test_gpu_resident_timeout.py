@@ -94,3 +94,46 @@ def test_contexts_without_a_counting_barrier_refuse_the_hook():
     S = _solver((48, 48, 48), "y", "f32", False)
     assert _status(lambda: S.set_barrier_test(0, 0)) == GLBE_ERR_ARG
     S.close()
+
+
+def test_every_synchronising_call_reports_until_a_state_is_set():
+    import torch
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_STATE, GLBE_ERR_TIMEOUT
+    calls = {"sync": lambda S: S.sync(), "residual": lambda S: S.residual(), "history": lambda S: S.history(),
+             "checkpoint": lambda S: S.checkpoint()}
+    S = _solver((48, 48, 48), "y", "f32c", True)
+    w = torch.ones(3, S.N, device="cuda")
+    for first in calls:
+        _start(S)
+        S.step(12)
+        _timed_out(S)
+        for name in (first, *calls):
+            assert _status(lambda: calls[name](S)) == GLBE_ERR_TIMEOUT, (first, name)
+        S.step(1)                             # also over a step launched by itself
+        assert _status(S.sync) == GLBE_ERR_TIMEOUT
+        for adjoint in (lambda: S.adjoint_steady(w, max_iters=20), lambda: S.adjoint_unrolled(4, 2, w)):
+            assert _status(adjoint) == GLBE_ERR_STATE
+    # not known to the host before the adjoint waits for the stream
+    _start(S)
+    _timed_out(S)
+    assert _status(lambda: S.adjoint_steady(w, max_iters=20)) == GLBE_ERR_STATE
+    _start(S)
+    for call in calls.values():
+        call(S)
+    S.close()
+
+
+def test_2d_every_synchronising_call_reports_until_a_state_is_set():
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
+    calls = {"sync": lambda S: S.sync(), "residual": lambda S: S.residual(), "history": lambda S: S.history()}
+    S = _solver2(True, "f32")
+    for first in calls:
+        _state2(S)
+        S.step(12)
+        _timed_out(S)
+        for name in (first, *calls):
+            assert _status(lambda: calls[name](S)) == GLBE_ERR_TIMEOUT, (first, name)
+    _state2(S)
+    for call in calls.values():
+        call(S)
+    S.close()
