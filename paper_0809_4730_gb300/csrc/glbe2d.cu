@@ -1664,6 +1664,7 @@ struct glbe2d_ctx {
     unsigned res_spin;      // polls of a barrier wait before it gives up
     int res_absent;         // block that leaves a march at once (failure test), or -1
     bool res_used;          // a resident march was launched since the error flag was last read
+    bool res_captured;      // a captured march may be replayed at any time: the flag is always read
     bool torn;              // a barrier wait ran out and no state was set since
 };
 
@@ -1862,6 +1863,7 @@ glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
     }
     GLBE2D_CUDA(e, "2D resident march");
     c->res_used = true;
+    if (stream_captures(c->stream)) c->res_captured = true;
     if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
     c->t += n;
     return GLBE_OK;
@@ -1872,7 +1874,7 @@ glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
 // march's stop flag.
 glbe_status sync_control2(glbe2d_ctx* c, int* stop)
 {
-    const bool resident = c->res_used && c->res.form >= 2;
+    const bool resident = (c->res_used || c->res_captured) && c->res.form >= 2;
     c->res_used = false;
     char* const base = reinterpret_cast<char*>(c->t_dev);   // start of the control words
     char misc[64] = {0};
@@ -2014,6 +2016,7 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
+    c->res_captured = false;
     c->torn = false;
     c->mass0 = p->rho0 * (double)fluid2(p);
     c->t = 0;

@@ -363,6 +363,7 @@ struct glbe_ctx {
     unsigned res_spin;       // polls of a barrier wait before it gives up
     int res_absent;          // block that leaves a march at once (failure test), or -1
     bool res_used;           // a resident march was launched since the error flag was last read
+    bool res_captured;       // a captured march may be replayed at any time: the flag is always read
     bool torn;               // a barrier wait ran out and no state was set since
     unsigned* sr_ctr;   // [2] seeds of stochastic rounding, read by the step of parity t & 1
     double mass0;   // rho0 x number of fluid nodes
@@ -473,6 +474,7 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
     }
     GLBE_CUDA(e, "resident march");
     c->res_used = true;
+    if (stream_captures(c->stream)) c->res_captured = true;
     if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
     c->t += n;
     return GLBE_OK;
@@ -484,7 +486,7 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
 // stream.  Every call that synchronises does it here.
 glbe_status sync_control(glbe_ctx* c, int* stop)
 {
-    const bool resident = c->res_used && c->res.form >= 2;
+    const bool resident = (c->res_used || c->res_captured) && c->res.form >= 2;
     c->res_used = false;
     char misc[64] = {0};
     if (stop || resident)
@@ -646,6 +648,7 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
+    c->res_captured = false;
     c->torn = false;
     c->mass0 = p->rho0 * (double)fluid_nodes(p);   // planes on walls and ghost planes excluded
     c->t = 0;

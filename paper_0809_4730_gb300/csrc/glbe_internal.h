@@ -279,6 +279,15 @@ __device__ __forceinline__ void grid_dependency_release() { asm volatile("gridde
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 
+// Whether work enqueued on the stream now is captured (or cannot be told not to be).
+inline bool stream_captures(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // What another translation unit (the adjoint) needs of a context: its
 // parameters and the buffers of the current time level t (the populations the
 // next step gathers from, the lagged Lorentz force, the force field).

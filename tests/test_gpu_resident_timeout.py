@@ -137,3 +137,34 @@ def test_2d_every_synchronising_call_reports_until_a_state_is_set():
     for call in calls.values():
         call(S)
     S.close()
+
+
+@pytest.mark.parametrize("two_d", [False, True])
+def test_replays_of_a_captured_march_are_checked(two_d):
+    """The wait runs out in replays alone: a synchronising call after the capture has found nothing."""
+    import torch
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        S = _solver2(True, "f32") if two_d else _solver((48, 48, 48), "y", "f32", True)
+        start = _state2 if two_d else _start
+        start(S)
+        S.step(20)
+        S.sync()
+        g = torch.cuda.CUDAGraph()
+        S.set_barrier_test(LIMIT, 0)
+        with torch.cuda.graph(g, stream=side):
+            S.step(20)
+        S.set_barrier_test(1 << 24, -1)
+        S.sync()
+        S.sync()
+        g.replay()
+        assert _status(S.sync) == GLBE_ERR_TIMEOUT
+        start(S)
+        S.sync()
+        g.replay()
+        assert _status(S.residual) == GLBE_ERR_TIMEOUT
+        start(S)
+        S.step(20)
+        S.sync()
+    S.close()
