@@ -197,10 +197,10 @@ glbe_status glbe_set_force_host(glbe_ctx* ctx, const float* h_F);
  * n >= 2 steps in one launch whose blocks stay resident and meet at a bounded
  * barrier between levels: the same states bit for bit.  Should a wait run out,
  * the state is incomplete: no such launch marches again and every call that
- * synchronises (glbe_sync, glbe_residual, glbe_history, glbe_checkpoint_save,
- * glbe_solve) returns GLBE_ERR_TIMEOUT, the adjoint calls, once it is known,
- * GLBE_ERR_STATE, until glbe_set_state or glbe_checkpoint_load gives the context
- * a state. */
+ * synchronises (glbe_sync, glbe_residual, glbe_history, glbe_checkpoint_save)
+ * returns GLBE_ERR_TIMEOUT, glbe_solve and the adjoint calls, whose own limit
+ * that status is, GLBE_ERR_STATE, until glbe_set_state or glbe_checkpoint_load
+ * gives the context a state. */
 glbe_status glbe_step_n(glbe_ctx* ctx, long n);
 
 /* Failure detection of those launches: a barrier wait gives up after
@@ -225,7 +225,8 @@ glbe_status glbe_history(glbe_ctx* ctx, glbe_residual_info* out, long cap, long*
  * launches, see glbe_step_n).  *steps_out = time
  * level t of the converged residual (or the level reached), *r_out = r(t).
  * GLBE_ERR_TIMEOUT if max_steps was reached first, GLBE_ERR_DIVERGED on
- * NaN/Inf.  Synchronises the stream. */
+ * NaN/Inf, GLBE_ERR_STATE (and *r_out = NaN) if a resident launch's barrier wait
+ * ran out.  Synchronises the stream. */
 glbe_status glbe_solve(glbe_ctx* ctx, double tol, long max_steps, long* steps_out, double* r_out);
 
 /* Macroscopic fields of the current state, as the next collision sees them

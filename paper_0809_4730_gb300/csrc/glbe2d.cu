@@ -2132,7 +2132,7 @@ glbe_status glbe2d_solve(glbe2d_ctx* c, double tol, long max_steps, long* steps_
             if (s != GLBE_OK) return s;
         }
         s = sync_control2(c, &stop);
-        if (s != GLBE_OK) return s;
+        if (s != GLBE_OK) return incomplete(s, r_out);
         if (stop) {
             glbe_residual_info info;
             const glbe_status rs = read_record2(c, &info);
@@ -2155,6 +2155,7 @@ glbe_status glbe2d_solve(glbe2d_ctx* c, double tol, long max_steps, long* steps_
     }
     glbe_residual_info info;
     s = read_record2(c, &info);
+    if (s == GLBE_ERR_TIMEOUT) return incomplete(s, r_out);
     if (steps_out) *steps_out = c->t;
     if (r_out) *r_out = info.t >= 0 ? info.r : NAN;
     if (s != GLBE_OK) return s;

@@ -26,7 +26,6 @@
 // adjoint writes them once and every iteration reads them in place of the
 // gathered state; the unrolled sweep, whose state changes every level,
 // gathers it.
-#include <cmath>
 #include <cstring>
 
 #include "glbe.h"
@@ -608,11 +607,7 @@ glbe_status glbe_adjoint_steady(glbe_ctx* ctx, const float* d_w, double tol, lon
     cudaGraphExecDestroy(exec);
     if (e != cudaSuccess) return fail(GLBE_ERR_CUDA, "adjoint iteration: %s", cudaGetErrorString(e));
     s = ctx_sync(ctx);
-    if (s == GLBE_ERR_TIMEOUT) {   // which means max_iters here
-        if (r_out) *r_out = NAN;
-        return fail(GLBE_ERR_STATE, "the state is incomplete: a barrier wait of the resident march ran out");
-    }
-    if (s != GLBE_OK) return s;
+    if (s != GLBE_OK) return incomplete(s, r_out);
     double rec[RECORD_STRIDE];
     ADJ_CUDA(cudaMemcpy(rec, record, sizeof rec, cudaMemcpyDeviceToHost), "adjoint record");
     if (iters_out) *iters_out = (long)rec[0];

@@ -536,7 +536,7 @@ size_t storage_value_bytes(int storage) { return storage_bytes(storage); }
 glbe_status ctx_view(glbe_ctx* c, CtxView* v)
 {
     if (!c || !v) return fail(GLBE_ERR_ARG, "ctx or view is NULL");
-    if (c->torn) return fail(GLBE_ERR_STATE, "the state is incomplete: a barrier wait of the resident march ran out");
+    if (c->torn) return incomplete(GLBE_ERR_TIMEOUT, nullptr);
     const int s = (int)(c->t & 1);
     v->prm = c->prm;
     v->sp = c->sp;
@@ -915,7 +915,7 @@ glbe_status glbe_solve(glbe_ctx* c, double tol, long max_steps, long* steps_out,
             if (s != GLBE_OK) return s;
         }
         s = sync_control(c, &stop);
-        if (s != GLBE_OK) return s;
+        if (s != GLBE_OK) return incomplete(s, r_out);
         if (stop) {
             glbe_residual_info info;
             glbe_status rs = read_record(c, &info);
@@ -939,6 +939,7 @@ glbe_status glbe_solve(glbe_ctx* c, double tol, long max_steps, long* steps_out,
     }
     glbe_residual_info info;
     s = read_record(c, &info);
+    if (s == GLBE_ERR_TIMEOUT) return incomplete(s, r_out);
     if (steps_out) *steps_out = c->t;
     if (r_out) *r_out = info.t >= 0 ? info.r : NAN;
     if (s != GLBE_OK) return s;

@@ -1,6 +1,7 @@
 // glbe_internal.h -- structures shared by the host side of the C-ABI
 // (glbe_api.cu) and the kernel translation units (glbe_step_*.cu).
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -278,6 +279,15 @@ cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned thre
 __device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
+
+// The status of a call whose GLBE_ERR_TIMEOUT is its own step or iteration limit,
+// for a synchronisation that found a timed-out march: *r_out is no residual then.
+inline glbe_status incomplete(glbe_status s, double* r_out)
+{
+    if (s != GLBE_ERR_TIMEOUT) return s;
+    if (r_out) *r_out = NAN;
+    return fail(GLBE_ERR_STATE, "the state is incomplete: a barrier wait of the resident march ran out");
+}
 
 // Whether work enqueued on the stream now is captured (or cannot be told not to be).
 inline bool stream_captures(cudaStream_t st)

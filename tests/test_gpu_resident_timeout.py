@@ -168,3 +168,25 @@ def test_replays_of_a_captured_march_are_checked(two_d):
         S.step(20)
         S.sync()
     S.close()
+
+
+@pytest.mark.parametrize("two_d", [False, True])
+def test_solve_does_not_pass_a_timed_out_wait_off_as_its_step_limit(two_d):
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_STATE, GLBE_ERR_TIMEOUT
+    S = _solver2(False, "f32") if two_d else _solver((48, 48, 48), "y", "f32", False)
+    start = _state2 if two_d else _start
+    # the wait runs out in the steps up to a residual level, in the solve's own march, and before the call
+    for before, cap in ((0, 400), (20, 400), (20, 7), (20, 0)):
+        start(S)
+        S.step(before)
+        S.set_barrier_test(LIMIT, 0)
+        if cap == 0:
+            S.step(5)
+        for _ in range(2):
+            assert _status(lambda: S.solve(1e-30, cap)) == GLBE_ERR_STATE
+        S.set_barrier_test(1 << 24, -1)
+        assert _status(lambda: S.solve(1e-30, cap)) == GLBE_ERR_STATE
+    start(S)
+    status, t, r = S.solve(1e-30, 40)
+    assert status == GLBE_ERR_TIMEOUT and t == 40 and r > 0
+    S.close()
