@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
     static_assert(!PAIR || (!MHD && !Store<ST>::COMP), "pairs: the flow step of the plain storage types");
     // the F32C coupled update needs over 128 registers in one pass
     constexpr int UNIT = PAIR ? (DENSE ? RES_PAIR : RES_NODE1) : DENSE && MHD && ST == ST_F32C ? RES_NODE2 : RES_NODE;
+    static_assert(RES_THREADS == 2 * PAIR_THREADS, "a tile of pairs is two launched blocks");
     extern __shared__ uint32_t slots[];          // [tile][RES_ROWS][blockDim.x]
     __shared__ float wsum[RES_THREADS / 32][RES_SUMS];
     __shared__ double bsum[RES_SUMS];
@@ -270,7 +271,7 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
             } else {
                 if (bounced != RES_SKIP)
                     resident_update<ST, MHD, MODE_STEP_RESID, UNIT>(p, b, i, tab, BT, bounced, acc);
-                // the tile's sums: FP32 within it as block_partials forms them, FP64 over the tiles
+                // the tile's sums: FP32 over the nodes of a launched block (see block_partials), FP64 from there on
 #pragma unroll
                 for (int r = 0; r < RES_SUMS; ++r) {
                     const float v = warp_sum(acc[r]);
@@ -279,7 +280,19 @@ __global__ void __launch_bounds__(RES_THREADS, DENSE ? resident_dense_blocks<ST,
                 __syncthreads();
                 if (threadIdx.x < RES_SUMS) {
                     float v = 0.f;
-                    for (int w = 0; w < BT / 32; ++w) v += wsum[w][threadIdx.x];
+                    if constexpr (UNIT == RES_PAIR) {
+                        // a tile is two launched blocks of pairs
+                        constexpr int GROUP = PAIR_THREADS / 32;
+                        float u = 0.f;
+#pragma unroll
+                        for (int w = 0; w < GROUP; ++w) {
+                            v += wsum[w][threadIdx.x];
+                            u += wsum[GROUP + w][threadIdx.x];
+                        }
+                        bsum[threadIdx.x] += (double)u;
+                    } else {
+                        for (int w = 0; w < BT / 32; ++w) v += wsum[w][threadIdx.x];
+                    }
                     bsum[threadIdx.x] += (double)v;
                 }
                 __syncthreads();
