@@ -199,8 +199,8 @@ glbe_status glbe_set_force_host(glbe_ctx* ctx, const float* h_F);
  * the state is incomplete: no such launch marches again and every call that
  * synchronises (glbe_sync, glbe_residual, glbe_history, glbe_checkpoint_save)
  * returns GLBE_ERR_TIMEOUT, glbe_solve and the adjoint calls, whose own limit
- * that status is, GLBE_ERR_STATE, until glbe_set_state or glbe_checkpoint_load
- * gives the context a state. */
+ * that status is, GLBE_ERR_STATE, until glbe_set_state (with every part of the
+ * state) or glbe_checkpoint_load gives the context a state. */
 glbe_status glbe_step_n(glbe_ctx* ctx, long n);
 
 /* Failure detection of those launches: a barrier wait gives up after

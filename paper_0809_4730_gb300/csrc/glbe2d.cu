@@ -2220,10 +2220,11 @@ glbe_status glbe2d_set_state(glbe2d_ctx* c, const float* d_df, const float* d_dg
         break;
     }
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state kernel");
+    const bool whole = !mhd || (d_dg && d_FL);   // makes good what a timed-out march left
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, ((long long)t + 9) / 10 * 10, c->stop_dev, 0, c->tol_dev, 0.0,
-                                         c->record, c->hist_count, 1, c->res_bar);
+                                         c->record, c->hist_count, 1, whole ? c->res_bar : nullptr);
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state reset");
-    c->torn = false;
+    if (whole) c->torn = false;
     return GLBE_OK;
 }
 

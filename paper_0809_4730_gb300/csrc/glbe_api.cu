@@ -993,11 +993,13 @@ glbe_status glbe_set_state(glbe_ctx* c, const float* d_df, const float* d_dg, co
     default: e = launch_set_state_t<ST_F32C>(mhd, c->sp, c->f[s], c->g[s], c->FL, d_df, d_dg, d_FL, c->stream); break;
     }
     GLBE_CUDA(e, "set_state kernel");
-    // a replaced state starts a fresh residual history
+    // a replaced state starts a fresh residual history; only a whole one makes
+    // good what a timed-out march left
+    const bool whole = d_df && (!mhd || (d_dg && d_FL));
     misc_set_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, (long long)t + 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record,
-                                            c->hist_count, 1, c->res_bar);
+                                            c->hist_count, 1, whole ? c->res_bar : nullptr);
     GLBE_CUDA(cudaGetLastError(), "set_state reset");
-    c->torn = false;
+    if (whole) c->torn = false;
     c->t = t;
     c->t_snap = -1;
     return GLBE_OK;

@@ -190,3 +190,27 @@ def test_solve_does_not_pass_a_timed_out_wait_off_as_its_step_limit(two_d):
     status, t, r = S.solve(1e-30, 40)
     assert status == GLBE_ERR_TIMEOUT and t == 40 and r > 0
     S.close()
+
+
+@pytest.mark.parametrize("two_d", [False, True])
+def test_a_part_of_a_state_does_not_make_up_for_a_timed_out_wait(two_d):
+    """Without dg or F_L those parts stay as the march left them, at different levels."""
+    from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
+    S = _solver2(True, "f32") if two_d else _solver((48, 48, 48), "y", "f32", True)
+    (_state2 if two_d else _start)(S)
+    df, dg, FL = S.get_state()
+    for part in ((df,), (df, dg), (df, None, FL)):
+        for reported in (True, False):
+            S.set_state(df, dg, FL)
+            S.sync()
+            _timed_out(S)
+            if reported:
+                assert _status(S.sync) == GLBE_ERR_TIMEOUT
+            S.set_state(*part)
+            S.step(12)
+            assert _status(S.sync) == GLBE_ERR_TIMEOUT
+    S.set_state(df, dg, FL)
+    S.set_state(df)                           # over a whole state a part is as good as ever
+    S.step(12)
+    S.sync()
+    S.close()
