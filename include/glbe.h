@@ -193,9 +193,13 @@ glbe_status glbe_set_force_host(glbe_ctx* ctx, const float* h_F);
 
 /* Advances n >= 0 time steps (one fused kernel per step; the residual is
  * evaluated inside the step that collides a level t with t % 10 == 0).  With
- * the automatic kernel form, small grids (up to about 350,000 nodes) take
- * n >= 2 steps in one launch whose blocks stay resident and meet at a bounded
- * barrier between levels: the same states bit for bit.  Should a wait run out,
+ * the automatic kernel form and the MRT collision, without box, lid or
+ * stochastic rounding, small grids take many steps in one launch whose blocks
+ * stay resident and meet at a bounded barrier between levels, the same states
+ * bit for bit: n >= 2 on up to 4096 nodes, n >= 5 on larger ones, up to about
+ * 310,000 nodes with induction (BF16, F16: 230,000), 350,000 without (BF16,
+ * F16: 190,000), and 620,000 (BF16, F16: 700,000) where nodes go in pairs (F32,
+ * BF16, F16; even nx, no walls on x).  Should a wait run out,
  * the state is incomplete: no such launch marches again and every call that
  * synchronises (glbe_sync, glbe_residual, glbe_history, glbe_checkpoint_save)
  * returns GLBE_ERR_TIMEOUT, glbe_solve and the adjoint calls, whose own limit

@@ -943,20 +943,29 @@ constexpr int dense2d_blocks()
 
 // ---------------------------------------------------------------------------
 // Resident march of small grids (glbe_resident_common.cuh): many steps in one
-// launch, one node per thread, the one-node kernel's arithmetic bit for bit.
+// launch, one node per thread and one tile per block, the one-node kernel's
+// arithmetic bit for bit.
 // Table rows: the source node of each D2Q9 direction (the node itself where
 // the link is bounced) and the bounced-link bits; the D2Q5 directions share
-// the sources of the axis directions.  A step takes (us, launched -> resident):
-//               F32 flow      F32 coupled   F32C coupled  BF16 coupled
-//   64 x 64     6.4 -> 1.7    6.6 -> 2.3    8.6 -> 3.0    6.7 -> 2.2
-//   128 x 128   6.5 -> 2.8    6.6 -> 3.5    8.5 -> 4.0    6.6 -> 3.2
-//   384 x 384   8.7 -> 5.9    8.9 -> 7.0   13.0 -> 10.9   8.9 -> 6.1
-// The line lies where the tables crowd out the gathers' L1: 820 x 820 coupled
-// F32 marched 29.5 us a step with 205 KB of tables on an SM and 24.3 launched,
-// 700 x 700 18.1 with 164 KB and 18.4 launched.
+// the sources of the axis directions.  One cluster (up to 4096 nodes) wins in
+// every form; past it only the coupled F32C grids of 8192 nodes and more do,
+// against launches that overlap (us a step, launched -> resident; in brackets
+// the cooperative forms that are not built):
+//               F32 flow        F32 coupled     F32C coupled    BF16 coupled
+//   64 x 64     2.5 -> 1.75     3.1 -> 2.4      3.9 -> 2.9      3.2 -> 2.0
+//   80 x 80     2.5 -> (3.1)    3.1 -> (3.5)    4.0 -> (4.0)    3.2 -> (3.3)
+//   128 x 128   2.7 -> (3.0)    3.6 -> (3.45)   5.3 -> 3.9      3.8 -> (3.3)
+//   192 x 192   3.6 -> (3.1)    5.3 -> (3.6)    5.6 -> 4.0      4.2 -> (3.4)
+//   384 x 384   5.1 -> (5.6)    5.9 -> (7.2)    8.4 -> (11.7)   5.3 -> (6.4)
+// and solves of 200 steps, whose launches a graph replays (us):
+//   80 x 80     583 -> (684)    668 -> (780)    838 -> (875)    710 -> (744)
+//   128 x 128   585 -> (681)    713 -> (775)    950 -> 868      688 -> (751)
+//   192 x 192   620 -> (707)    787 -> (802)   1111 -> 879      827 -> (755)
+// (past 38,912 nodes, one tile on each SM, F32C coupled solves gained 1 to 4 %
+// up to 256 x 256 and lost 11 % at 288 x 288).
 // ---------------------------------------------------------------------------
 constexpr int RES2_ROWS = 10;
-constexpr size_t RES2_TABLES = (size_t)16 * RES2_ROWS * 256 * 4;   // table bytes of an SM, at most
+constexpr uint32_t RES2_LEAST = 8192;     // nodes of the cooperative form, at least
 __host__ __device__ constexpr int axis9(int a5) { return a5 == 0 ? 0 : (a5 == 1 ? 1 : (a5 == 2 ? 3 : (a5 == 3 ? 2 : 4))); }
 static_assert(ex9(axis9(2)) == ex5(2) && ey9(axis9(3)) == ey5(3), "D2Q5 directions among the D2Q9 ones");
 
@@ -1023,36 +1032,33 @@ __device__ __forceinline__ void resident_update2(const P2& p, const B2& b, int n
     node2_from_sources<ST, MHD, MODE>(p, b, o, n, d, dl, q, ql, us, acc);
 }
 
-// DENSE: several tiles a block, held to the register budgets of the launched
-// plain steps (BF16 coupled: free there, four blocks here).
 // Residual sums: a warp's FP32 sums, those of GROUP warps added in order (the
 // partial of a launched block), and from there on FP64: in the cluster form in
-// the launched reduction's order, in the others a block's partials first, so
+// the launched reduction's order, in the other a block's partials first, so
 // that a level's sums are one number per block.
-template <int ST, bool MHD, bool DENSE, bool CLUSTER>
-__global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, MHD>() ? dense2d_blocks<ST, MHD>() : 4)
-    resident2d_kernel(const P2 p, const ResidentMarch m)
+template <int ST, bool MHD, bool CLUSTER>
+__global__ void __launch_bounds__(RES_THREADS, 1) resident2d_kernel(const P2 p, const ResidentMarch m)
 {
     constexpr int GROUP = T2D / 32;
-    extern __shared__ uint32_t slots[];          // [tile][RES2_ROWS][blockDim.x]
-    // warp sums: of the block's tile, or of the whole grid (CLUSTER)
+    extern __shared__ uint32_t slots[];          // [RES2_ROWS][blockDim.x]
+    // warp sums: of the block, or of the whole grid (CLUSTER)
     __shared__ float wsum[RES_SUMS][CLUSTER ? RES_CLUSTER * RES_THREADS / 32 : RES_THREADS / 32];
-    __shared__ double bsum[RES_SUMS], tot[RES_SUMS];   // of the block's tiles; of the grid
+    __shared__ double tot[RES_SUMS];             // the grid's sums
     __shared__ int verdict;
     const int BT = blockDim.x, G = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = BT >> 5;
     if (m.solve && *(volatile int*)m.out.stop) return;   // converged in an earlier launch
     if (!CLUSTER && (int)blockIdx.x == m.absent) return;
-    const uint32_t ntiles = ((uint32_t)p.N + BT - 1) / BT;
-    int mine = 0;
-    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, ++mine)
-        resident_slots2(p, tile * BT + threadIdx.x, slots + (size_t)mine * RES2_ROWS * BT + threadIdx.x, BT);
+    const int n = (int)blockIdx.x * BT + (int)threadIdx.x;
+    uint32_t* const tab = slots + threadIdx.x;
+    resident_slots2(p, (uint32_t)n, tab, BT);
+    const unsigned flags = tab[(RES2_ROWS - 1) * BT];
     if constexpr (CLUSTER) {
         for (int i = threadIdx.x; i < RES_SUMS * RES_CLUSTER * RES_THREADS / 32; i += BT) (&wsum[0][0])[i] = 0.f;
         cluster_level_barrier();                 // every block's shared memory is there to write to
     }
     unsigned gen = 0;
     if (!CLUSTER && threadIdx.x == 0) gen = *(volatile unsigned*)(m.bar + 1);
-    const bool writer = blockIdx.x == G - 1;    // the last block has no more tiles than any other
+    const bool writer = blockIdx.x == G - 1;
     B2 b{};
     b.FL = m.FL;
     b.Ffield = m.Ffield;
@@ -1066,50 +1072,43 @@ __global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, M
         b.gsrc = m.g[par];
         b.gdst = m.g[par ^ 1];
         b.have_snap = snap ? 1 : 0;
-        if (!CLUSTER && resid && threadIdx.x < RES_SUMS) bsum[threadIdx.x] = 0.0;
-        for (int k = 0; k < mine; ++k) {
-            const uint32_t tile = blockIdx.x + (uint32_t)k * G;
-            const uint32_t* tab = slots + (size_t)k * RES2_ROWS * BT + threadIdx.x;
-            const unsigned flags = tab[(RES2_ROWS - 1) * BT];
-            float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (!resid) {
-                if (flags != RES_SKIP)
-                    resident_update2<ST, MHD, M2_STEP>(p, b, (int)(tile * BT + threadIdx.x), tab, BT, flags, acc);
+        float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (flags != RES_SKIP) {
+            if (resid) resident_update2<ST, MHD, M2_RESID>(p, b, n, tab, BT, flags, acc);
+            else resident_update2<ST, MHD, M2_STEP>(p, b, n, tab, BT, flags, acc);
+        }
+        const bool sums = resid && snap;
+        if (sums) {
+#pragma unroll
+            for (int r = 0; r < RES_SUMS; ++r) acc[r] = warp_sum(acc[r]);
+            if constexpr (CLUSTER) {
+                // into every block's shared memory
+                const int at = (int)blockIdx.x * warps + warp;
+#pragma unroll
+                for (int r = 0; r < RES_SUMS; ++r) acc[r] = __shfl_sync(0xffffffffu, acc[r], 0);
+                if (lane < G) {
+                    auto cl = cooperative_groups::this_cluster();
+#pragma unroll
+                    for (int r = 0; r < RES_SUMS; ++r) *cl.map_shared_rank(&wsum[r][at], lane) = acc[r];
+                }
             } else {
-                if (flags != RES_SKIP)
-                    resident_update2<ST, MHD, M2_RESID>(p, b, (int)(tile * BT + threadIdx.x), tab, BT, flags, acc);
-                if (!snap) continue;
+                if (lane == 0) {
 #pragma unroll
-                for (int r = 0; r < RES_SUMS; ++r) acc[r] = warp_sum(acc[r]);
-                if constexpr (CLUSTER) {
-                    // into every block's shared memory
-                    const int at = (int)tile * warps + warp;
+                    for (int r = 0; r < RES_SUMS; ++r) wsum[r][warp] = acc[r];
+                }
+                __syncthreads();
+                if (threadIdx.x < RES_SUMS) {
+                    double t = 0.0;
+                    for (int q = 0; q < warps; q += GROUP) {
+                        float v = 0.f;
 #pragma unroll
-                    for (int r = 0; r < RES_SUMS; ++r) acc[r] = __shfl_sync(0xffffffffu, acc[r], 0);
-                    if (lane < G) {
-                        auto cl = cooperative_groups::this_cluster();
-#pragma unroll
-                        for (int r = 0; r < RES_SUMS; ++r) *cl.map_shared_rank(&wsum[r][at], lane) = acc[r];
+                        for (int w = 0; w < GROUP; ++w) v += wsum[threadIdx.x][q + w];
+                        t += (double)v;
                     }
-                } else {
-                    if (lane == 0) {
-#pragma unroll
-                        for (int r = 0; r < RES_SUMS; ++r) wsum[r][warp] = acc[r];
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < RES_SUMS) {
-                        for (int q = 0; q < warps; q += GROUP) {
-                            float v = 0.f;
-#pragma unroll
-                            for (int w = 0; w < GROUP; ++w) v += wsum[threadIdx.x][q + w];
-                            bsum[threadIdx.x] += (double)v;
-                        }
-                    }
-                    __syncthreads();
+                    m.partials[(size_t)threadIdx.x * G + blockIdx.x] = t;
                 }
             }
         }
-        const bool sums = resid && snap;
         if constexpr (CLUSTER) {
             cluster_level_barrier();
             if (sums) {
@@ -1126,7 +1125,6 @@ __global__ void __launch_bounds__(RES_THREADS, !DENSE ? 1 : dense2d_blocks<ST, M
                 }
             }
         } else {
-            if (sums && threadIdx.x < RES_SUMS) m.partials[(size_t)threadIdx.x * G + blockIdx.x] = bsum[threadIdx.x];
             if (!resident_barrier(m.bar, gen, m.spin_limit)) return;
             if (sums && (m.solve || writer)) {
                 // a solve's blocks all take the decision (num, den, non-finite count), from the same numbers in
@@ -1158,15 +1156,21 @@ template <int ST, bool MHD>
 cudaError_t resident2d_plan_t(uint32_t N, ResidentPlan* out)
 {
     constexpr size_t tile = (size_t)RES2_ROWS * RES_THREADS * sizeof(uint32_t);
-    auto* cluster = resident2d_kernel<ST, MHD, false, true>;
-    auto* free_form = resident2d_kernel<ST, MHD, false, false>;
-    auto* dense = resident2d_kernel<ST, MHD, true, false>;
-    static const ResidentOcc of = resident_occupancy(free_form, tile), od = resident_occupancy(dense, tile);
+    using K = void (*)(P2, ResidentMarch);
+    const K cluster = resident2d_kernel<ST, MHD, true>;
+    K coop = nullptr;
+    ResidentOcc oc{};
+    if constexpr (ST == GLBE_F32C && MHD) {
+        coop = resident2d_kernel<ST, MHD, false>;
+        static const ResidentOcc occ = resident_occupancy(coop, tile);
+        if (N >= RES2_LEAST) oc = occ;
+    }
     static const bool fits = [&] {
         cudaFuncSetAttribute(cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return resident_cluster_fits(cluster, tile);
     }();
-    return resident_plan_of(cluster, free_form, dense, N, N, RES2_ROWS, RES2_TABLES, of, od, fits, out);
+    return resident_plan_of(cluster, coop, K(nullptr), N, N, RES2_ROWS, RES_MAX_TILES * tile, oc, ResidentOcc{}, fits,
+                            out);
 }
 
 template <int ST>
@@ -1175,18 +1179,14 @@ cudaError_t resident2d_plan(bool mhd, uint32_t N, ResidentPlan* out)
     return mhd ? resident2d_plan_t<ST, true>(N, out) : resident2d_plan_t<ST, false>(N, out);
 }
 
-template <int ST, bool MHD>
-cudaError_t resident2d_march_t(const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
-{
-    if (pl.form == 1) return resident_launch(resident2d_kernel<ST, MHD, false, true>, pl, st, p, m);
-    if (pl.form == 2) return resident_launch(resident2d_kernel<ST, MHD, false, false>, pl, st, p, m);
-    return resident_launch(resident2d_kernel<ST, MHD, true, false>, pl, st, p, m);
-}
-
 template <int ST>
 cudaError_t resident2d_march(bool mhd, const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
 {
-    return mhd ? resident2d_march_t<ST, true>(p, m, pl, st) : resident2d_march_t<ST, false>(p, m, pl, st);
+    if constexpr (ST == GLBE_F32C) {
+        if (pl.form == 2) return resident_launch(resident2d_kernel<ST, true, false>, pl, st, p, m);
+    }
+    return mhd ? resident_launch(resident2d_kernel<ST, true, true>, pl, st, p, m)
+               : resident_launch(resident2d_kernel<ST, false, true>, pl, st, p, m);
 }
 
 // Two x-adjacent nodes per thread (x periodic, even nx; FP32 or BF16
@@ -2050,7 +2050,7 @@ glbe_status glbe2d_step_n(glbe2d_ctx* c, long n)
 {
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(GLBE_ERR_ARG, "n must be >= 0");
-    if (c->res.form && n >= 2) {
+    if (resident_takes(c->res, n)) {
         for (long k = 0; k < n; k += RES_MOST_STEPS) {
             const glbe_status s = enqueue_resident2(c, n - k < RES_MOST_STEPS ? n - k : RES_MOST_STEPS, false, 0.0);
             if (s != GLBE_OK) return s;

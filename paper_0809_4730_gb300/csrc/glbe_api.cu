@@ -750,7 +750,7 @@ glbe_status glbe_step_n(glbe_ctx* c, long n)
     NvtxRange range_("glbe_step_n");
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(GLBE_ERR_ARG, "n must be >= 0");
-    if (c->res.form && n >= 2) {
+    if (resident_takes(c->res, n)) {
         for (long k = 0; k < n; k += RES_MOST_STEPS) {
             const glbe_status s = enqueue_resident(c, n - k < RES_MOST_STEPS ? n - k : RES_MOST_STEPS, false, 0.0);
             if (s != GLBE_OK) return s;

@@ -219,6 +219,12 @@ struct ResidentPlan {
     int blocks, threads;
     unsigned smem;
 };
+// Whether n steps are marched so.  A cooperative launch, its tables and the look
+// at its flag when the host next waits cost as much as some four launched steps
+// save: two F32 steps of 64^3 and a wait took 57 us so and 45 launched, four 75
+// and 63, eight 111 and 105 (40^3: 47 and 36, 55 and 46, 72 and 72); a cluster's
+// two steps cost what two launched ones do (4 x 32 x 4: 37 and 36 us).
+inline bool resident_takes(const ResidentPlan& pl, long n) { return pl.form == 1 ? n >= 2 : pl.form && n >= 5; }
 template <int ST>
 cudaError_t resident_plan(bool mhd, const StepParams& p, ResidentPlan* out);
 template <int ST>

@@ -2,18 +2,23 @@
 // (glbe_resident_common.cuh): the gather tables, node updates and launch forms.
 //
 // A grid of at most a few nodes per resident thread is not bound by memory: a
-// launched step takes 8.5 us on every grid of up to 48^3 nodes (F32, flow),
+// launched step takes 4 to 6 us on every grid of up to 40^3 nodes (F32, flow),
 // most of it the launch itself, kernel prologue, geometry and the latency of
-// one gather.  Resident, a step takes (us, launched before -> resident):
-//                 F32 flow      F32 coupled   F32C flow     F32C coupled
-//   4 x 32 x 4    8.5 -> 1.9    8.5 -> 2.6    8.5 -> 1.6    10.0 -> 3.5
-//   64 x 64 x 8   8.7 -> 3.9    8.7 -> 4.6    8.5 -> 4.0    10.5 -> 5.7
-//   40^3          8.8 -> 4.4   10.8 -> 6.4   10.6 -> 5.6    14.6 -> 9.0
-//   64^3         13.2 -> 9.4   21.5 -> 17.5  17.7 -> 15.2   37.9 -> 30.4
-// (launched: with the reduction of glbe_residual.cuh).  The line lies where
-// the tables crowd out the gathers' L1 (RES_TABLES_FLOW, RES_TABLES_MHD):
-// 72^3 coupled marched 32.7 us a step with 205 KB of tables on an SM, 29.5
-// launched (F32C 56.3 and 52.7).  The node update is the step kernels'
+// one gather.  A step of long marches takes (us, launched with overlap ->
+// resident):
+//            F32 flow       F32 coupled    F32C flow      F32C coupled   BF16 flow
+//   16^3     4.1 -> 2.1     4.5 -> 2.9     4.6 -> 1.95    5.7 -> 3.9     4.2 -> 1.8
+//   32^3     5.0 -> 3.6     6.0 -> 4.1     6.3 -> 3.8     6.2 -> 5.2     4.5 -> 3.4
+//   40^3     5.7 -> 4.4     7.2 -> 6.2     7.3 -> 5.5    10.1 -> 8.8     5.9 -> 3.7
+//   64^3     9.2 -> 8.8    17.8 -> 16.4   13.9 -> 12.65  31.9 -> 27.8    6.95 -> 6.9
+//   80^3    15.9 -> 13.6        -              -              -         11.45 -> 9.8
+//   84^3    18.8 -> 16.3        -              -              -         12.3 -> 10.7
+// The line lies where the tables crowd out the gathers' L1 (RES_TABLES_FLOW,
+// RES_TABLES_MHD) or the SM is full: pairs (flow, even nx, x periodic) march to
+// 622,592 nodes in F32 and 700,416 in the 16-bit forms, one node a thread to
+// 350,208 (F32, F32C; 16 bits 194,560), coupled ones to 311,296 (16 bits
+// 233,472) on 152 SMs.  72^3 coupled marched 32.7 us a step with 205 KB of
+// tables on an SM, 27.1 launched (F32C 56.3 and 44.8).  The node update is the step kernels'
 // (node_from_sources, pair_from_sources), so the states are theirs bit for bit.
 #pragma once
 #include <type_traits>
@@ -23,9 +28,9 @@
 namespace glbe {
 
 constexpr int RES_ROWS = 20;            // table rows: 19 slots and a flag word
-// Table bytes of an SM, at most: 9 tiles (64^3 F32C flow: 15.4 us a step with
-// them, 17.7 launched), 8 where a coupled node gathers f twice (64^3 F32C: 31
-// and 37.9 us; with 10 tiles the launched step is faster).
+// Table bytes of an SM, at most: 9 tiles (70^3 F32C flow: 16.3 us a step with
+// them, 17.2 launched), 8 where a coupled node gathers f twice (64^3 F32C: 27.8
+// and 31.9 us; with 10 tiles the launched step is faster).
 constexpr size_t RES_TABLES_FLOW = (size_t)9 * RES_ROWS * 256 * 4, RES_TABLES_MHD = (size_t)8 * RES_ROWS * 256 * 4;
 
 // Slots of node i's gather in column tid of the table: row a holds the index

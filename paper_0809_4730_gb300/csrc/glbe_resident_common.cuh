@@ -151,6 +151,7 @@ inline bool resident_grid_plan(const ResidentOcc& occ, uint32_t units, int sms, 
                                size_t table_bytes, int form, ResidentPlan* out)
 {
     const uint32_t tiles = (units + RES_THREADS - 1) / RES_THREADS;
+    if (occ.n[1] < 1) return false;
     for (int per = 1; per <= max_per && occ.n[per] == occ.n[1] && occ.n[1] * per * tile_bytes <= table_bytes; ++per) {
         const long long room = (long long)occ.n[1] * sms;
         if (room * per < tiles) continue;
@@ -164,6 +165,7 @@ inline bool resident_grid_plan(const ResidentOcc& occ, uint32_t units, int sms, 
 // block (registers unbounded), several tiles a block (held to the register
 // budget of the launched steps).  units_dense: updates of the dense form.
 // The attributes set are the device's: the same values whoever sets them.
+// A form with a null kernel and no occupancy is left out.
 template <class C, class K>
 cudaError_t resident_plan_of(C cluster, K free_form, K dense, uint32_t N, uint32_t units_dense, int rows,
                              size_t table_bytes, const ResidentOcc& occ_free, const ResidentOcc& occ_dense, bool cluster_fits,

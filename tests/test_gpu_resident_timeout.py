@@ -26,12 +26,11 @@ def _timed_out(S, absent=0):
     S.set_barrier_test(1 << 24, -1)
 
 
-def _solver2(mhd, storage, shape=(128, 304)):
+def _solver2(shape=(128, 300), **kw):
     from paper_0809_4730_gb300.glbe import Solver2D
-    kw = dict(wall_lo=(0, 1), wall_hi=(0, 1), gamma=0.2, nu=0.05, F=(2e-6, 1e-6), storage=storage)
-    if mhd:
-        kw.update(induction=1, gamma_m=0.2, eta=0.05, chi=0.05, mu=1.0, B0=(0.002, 0.004))
-    return Solver2D(*shape, **kw)
+    return Solver2D(*shape, wall_lo=(0, 1), wall_hi=(0, 1), gamma=0.2, nu=0.05, F=(2e-6, 1e-6),
+                    **dict(dict(storage="f32c", induction=1, gamma_m=0.2, eta=0.05, chi=0.05, mu=1.0, B0=(0.002, 0.004)),
+                           **kw))
 
 
 def _state2(S):
@@ -66,10 +65,9 @@ def test_a_new_state_marches_as_before(shape, storage, mhd, reported):
     B.close()
 
 
-@pytest.mark.parametrize("storage,mhd", [("f32", False), ("f32c", True)])
-def test_2d_a_new_state_marches_as_before(storage, mhd):
+def test_2d_a_new_state_marches_as_before():
     from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
-    A, B = _solver2(mhd, storage), _solver2(mhd, storage)
+    A, B = _solver2(), _solver2()
     _state2(B)
     for _ in range(23):
         B.step(1)
@@ -126,7 +124,7 @@ def test_every_synchronising_call_reports_until_a_state_is_set():
 def test_2d_every_synchronising_call_reports_until_a_state_is_set():
     from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
     calls = {"sync": lambda S: S.sync(), "residual": lambda S: S.residual(), "history": lambda S: S.history()}
-    S = _solver2(True, "f32")
+    S = _solver2()
     for first in calls:
         _state2(S)
         S.step(12)
@@ -146,7 +144,7 @@ def test_replays_of_a_captured_march_are_checked(two_d):
     from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
     side = torch.cuda.Stream()
     with torch.cuda.stream(side):
-        S = _solver2(True, "f32") if two_d else _solver((48, 48, 48), "y", "f32", True)
+        S = _solver2() if two_d else _solver((48, 48, 48), "y", "f32", True)
         start = _state2 if two_d else _start
         start(S)
         S.step(20)
@@ -173,7 +171,7 @@ def test_replays_of_a_captured_march_are_checked(two_d):
 @pytest.mark.parametrize("two_d", [False, True])
 def test_solve_does_not_pass_a_timed_out_wait_off_as_its_step_limit(two_d):
     from paper_0809_4730_gb300.glbe import GLBE_ERR_STATE, GLBE_ERR_TIMEOUT
-    S = _solver2(False, "f32") if two_d else _solver((48, 48, 48), "y", "f32", False)
+    S = _solver2() if two_d else _solver((48, 48, 48), "y", "f32", False)
     start = _state2 if two_d else _start
     # the wait runs out in the steps up to a residual level, in the solve's own march, and before the call
     for before, cap in ((0, 400), (20, 400), (20, 7), (20, 0)):
@@ -196,7 +194,7 @@ def test_solve_does_not_pass_a_timed_out_wait_off_as_its_step_limit(two_d):
 def test_a_part_of_a_state_does_not_make_up_for_a_timed_out_wait(two_d):
     """Without dg or F_L those parts stay as the march left them, at different levels."""
     from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
-    S = _solver2(True, "f32") if two_d else _solver((48, 48, 48), "y", "f32", True)
+    S = _solver2() if two_d else _solver((48, 48, 48), "y", "f32", True)
     (_state2 if two_d else _start)(S)
     df, dg, FL = S.get_state()
     for part in ((df,), (df, dg), (df, None, FL)):
