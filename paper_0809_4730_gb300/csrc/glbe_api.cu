@@ -767,7 +767,8 @@ glbe_status glbe_step_n(glbe_ctx* c, long n)
 glbe_status glbe_sync(glbe_ctx* c)
 {
     if (!c) return fail(GLBE_ERR_ARG, "ctx is NULL");
-    GLBE_CUDA(cudaStreamSynchronize(c->stream), "glbe_sync");
+    const glbe_status s = sync_control(c, nullptr);   // the one wait for the stream
+    if (s != GLBE_OK) return s;
     int waited_out = 0;
     switch (c->prm.storage) {
     case GLBE_F32: waited_out = tile_wait_error_t<ST_F32>(); break;
@@ -776,7 +777,7 @@ glbe_status glbe_sync(glbe_ctx* c)
     default: break;
     }
     if (waited_out) return fail(GLBE_ERR_TIMEOUT, "a pipeline wait of the TMA-staged step kernel ran out");
-    return sync_control(c, nullptr);
+    return GLBE_OK;
 }
 
 glbe_status glbe_set_barrier_test(glbe_ctx* c, long long spin_limit, int absent_block)
