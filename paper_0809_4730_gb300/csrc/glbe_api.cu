@@ -234,7 +234,7 @@ StepParams glbe::make_step_params(const glbe_params* p)
     // an x axis without walls the whole axis, since the gather corrects the
     // sources that cross the x seam (a warp covers x-consecutive nodes, so
     // the seam nodes would otherwise split their warps between two paths)
-    s.interior_ok = 1;
+    s.interior_ok = !s.cavity;   // the cavity kernels gather every node alike
     const int n[3] = {p->nx, p->ny, p->nz};
     for (int d = 0; d < 3; ++d) {
         int lo = 1 + p->wall_lo[d], hi = n[d] - 2 - p->wall_hi[d];
@@ -242,23 +242,6 @@ StepParams glbe::make_step_params(const glbe_params* p)
         if (hi < lo) s.interior_ok = 0;
         s.ilo[d] = (uint32_t)lo;
         s.ispan[d] = hi >= lo ? (uint32_t)(hi - lo) : 0u;
-    }
-    if (s.cavity) {
-        // interior nodes of a cavity: inside the box with a margin of one node
-        // (no bounced link, none to the lid); on an axis the box spans whole
-        // without walls the periodic-seam rule of the plain grid stays
-        const int n[3] = {p->nx, p->ny, p->nz};
-        s.interior_ok = 1;
-        for (int d = 0; d < 3; ++d) {
-            if (p->box && p->box_lo[d] == 0 && p->box_hi[d] == n[d] - 1 && !p->wall_lo[d] && !p->wall_hi[d]) continue;
-            int lo = (p->box ? p->box_lo[d] : 0) + 1, hi = (p->box ? p->box_hi[d] : n[d] - 1) - 1;
-            if (lo < 1 + p->wall_lo[d]) lo = 1 + p->wall_lo[d];
-            if (hi > n[d] - 2 - p->wall_hi[d]) hi = n[d] - 2 - p->wall_hi[d];
-            if (d == 2 && hi > s.top_z - 1) hi = s.top_z - 1;
-            if (hi < lo) s.interior_ok = 0;
-            s.ilo[d] = (uint32_t)lo;
-            s.ispan[d] = hi >= lo ? (uint32_t)(hi - lo) : 0u;
-        }
     }
     // D3Q19 directions in the order of include/glbe.h
     static const int E[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
