@@ -1863,7 +1863,7 @@ glbe_status enqueue_resident2(glbe2d_ctx* c, long n, bool solve, double tol)
     }
     GLBE2D_CUDA(e, "2D resident march");
     c->res_used = true;
-    if (stream_captures(c->stream)) c->res_captured = true;
+    if (c->res.form >= 2 && stream_captures(c->stream)) c->res_captured = true;
     if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
     c->t += n;
     return GLBE_OK;
@@ -2012,7 +2012,7 @@ glbe_status glbe2d_init(const glbe2d_params* p, void* d_workspace, size_t bytes,
     c->tol_dev = reinterpret_cast<double*>(misc + 16);
     c->stop_dev = reinterpret_cast<int*>(misc + 24);
     c->res_bar = reinterpret_cast<unsigned*>(misc + 32);
-    c->res = plan_resident2(c);
+    c->res = stream_is_partitioned(static_cast<cudaStream_t>(p->stream)) ? ResidentPlan{} : plan_resident2(c);
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
@@ -2222,7 +2222,7 @@ glbe_status glbe2d_set_state(glbe2d_ctx* c, const float* d_df, const float* d_dg
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state kernel");
     const bool whole = !mhd || (d_dg && d_FL);   // makes good what a timed-out march left
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, ((long long)t + 9) / 10 * 10, c->stop_dev, 0, c->tol_dev, 0.0,
-                                         c->record, c->hist_count, 1, whole ? c->res_bar : nullptr);
+                                         c->record, c->hist_count, 1, whole && c->res.form >= 2 ? c->res_bar : nullptr);
     GLBE2D_CUDA(cudaGetLastError(), "2D set_state reset");
     if (whole) c->torn = false;
     return GLBE_OK;

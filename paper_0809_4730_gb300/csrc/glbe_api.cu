@@ -4,6 +4,8 @@
 // into the two population buffers (ping-pong of the pull scheme), the lagged
 // Lorentz force, the body-force field, the velocity snapshot of the residual,
 // per-block FP64 partial sums and a small record/history area.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -457,7 +459,7 @@ glbe_status enqueue_resident(glbe_ctx* c, long n, bool solve, double tol)
     }
     GLBE_CUDA(e, "resident march");
     c->res_used = true;
-    if (stream_captures(c->stream)) c->res_captured = true;
+    if (c->res.form >= 2 && stream_captures(c->stream)) c->res_captured = true;
     if (first < c->t + n) c->t_snap = (c->t + n - 1) / 10 * 10;
     c->t += n;
     return GLBE_OK;
@@ -536,6 +538,25 @@ glbe_status ctx_view(glbe_ctx* c, CtxView* v)
 }
 
 glbe_status ctx_sync(glbe_ctx* c) { return sync_control(c, nullptr); }
+
+bool stream_is_partitioned(cudaStream_t st)
+{
+    // through the runtime's driver entry point, as in glbe_noalloc.cu; a driver
+    // without it has no green contexts
+    using Fn = CUresult (*)(CUstream, CUgreenCtx*);
+    static const Fn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &f, 12040, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            f = nullptr;
+            cudaGetLastError();
+        }
+        return reinterpret_cast<Fn>(f);
+    }();
+    CUgreenCtx g = nullptr;
+    return fn && fn(st, &g) == CUDA_SUCCESS && g != nullptr;
+}
 
 cudaError_t launch_finalize(double* partials, unsigned nblocks, double mass0, long long* t_dev, double* record,
                             double* hist, unsigned long long* hist_count, unsigned hist_cap, int* stop,
@@ -627,7 +648,7 @@ glbe_status glbe_init(const glbe_params* p, void* d_workspace, size_t bytes, glb
     c->stop_dev = reinterpret_cast<int*>(misc + 24);
     c->sr_ctr = reinterpret_cast<unsigned*>(misc + 32);
     c->res_bar = reinterpret_cast<unsigned*>(misc + 40);
-    c->res = plan_resident(c);
+    c->res = stream_is_partitioned(static_cast<cudaStream_t>(p->stream)) ? ResidentPlan{} : plan_resident(c);
     c->res_spin = RES_SPIN_LIMIT;
     c->res_absent = -1;
     c->res_used = false;
@@ -981,7 +1002,7 @@ glbe_status glbe_set_state(glbe_ctx* c, const float* d_df, const float* d_dg, co
     // good what a timed-out march left
     const bool whole = d_df && (!mhd || (d_dg && d_FL));
     misc_set_kernel<<<1, 1, 0, c->stream>>>(c->t_dev, (long long)t + 10, c->stop_dev, 0, c->tol_dev, 0.0, c->record,
-                                            c->hist_count, 1, whole ? c->res_bar : nullptr);
+                                            c->hist_count, 1, whole && c->res.form >= 2 ? c->res_bar : nullptr);
     GLBE_CUDA(cudaGetLastError(), "set_state reset");
     if (whole) c->torn = false;
     c->t = t;

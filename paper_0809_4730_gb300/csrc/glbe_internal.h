@@ -295,6 +295,11 @@ inline glbe_status incomplete(glbe_status s, double* r_out)
     return fail(GLBE_ERR_STATE, "the state is incomplete: a barrier wait of the resident march ran out");
 }
 
+// Whether the stream belongs to a green context, a part of the device's SMs.  A
+// resident march is planned for all of them (a cooperative launch over every SM,
+// a cluster across 16), so there steps are launched one by one.
+bool stream_is_partitioned(cudaStream_t st);
+
 // Whether work enqueued on the stream now is captured (or cannot be told not to be).
 inline bool stream_captures(cudaStream_t st)
 {
