@@ -226,8 +226,8 @@ glbe_status glbe_history(glbe_ctx* ctx, glbe_residual_info* out, long cap, long*
 
 /* Time-marches until r(t) <= tol (t a multiple of 10) or max_steps steps have
  * been taken, replaying a CUDA graph of 10-step chunks (small grids: resident
- * launches, see glbe_step_n).  *steps_out = time
- * level t of the converged residual (or the level reached), *r_out = r(t).
+ * launches, see glbe_step_n).  *steps_out = time level t of the converged
+ * residual (or the level reached), *r_out = r(t).
  * GLBE_ERR_TIMEOUT if max_steps was reached first, GLBE_ERR_DIVERGED on
  * NaN/Inf, GLBE_ERR_STATE (and *r_out = NaN) if a resident launch's barrier wait
  * ran out.  Synchronises the stream. */

@@ -126,9 +126,9 @@ glbe_status glbe2d_history(glbe2d_ctx* ctx, glbe_residual_info* out, long cap, l
 
 /* Marches until r(t) <= tol at a level t that is a multiple of 10, or until
  * max_steps steps were taken, replaying a CUDA graph of 10-step chunks whose
- * kernels stop on a device flag (small grids: resident launches).  *steps_out = the converged level (or the
- * level reached), *r_out = its r.  GLBE_ERR_TIMEOUT / GLBE_ERR_DIVERGED as
- * glbe_solve.  Syncs. */
+ * kernels stop on a device flag (small grids: resident launches).  *steps_out =
+ * the converged level (or the level reached), *r_out = its r.
+ * GLBE_ERR_TIMEOUT / GLBE_ERR_DIVERGED / GLBE_ERR_STATE as glbe_solve.  Syncs. */
 glbe_status glbe2d_solve(glbe2d_ctx* ctx, double tol, long max_steps, long* steps_out, double* r_out);
 
 /* Fields of the current state as the next collision sees them: d_rho [N],

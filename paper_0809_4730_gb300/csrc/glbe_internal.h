@@ -264,7 +264,7 @@ StepParams make_step_params(const glbe_params* p);
 // coherent loads only.  What is hidden is the launch and the first blocks' set-up, 2 to 4 us
 // a step: ten coupled F32 steps on 128^3 with fields 1297 -> 1263 us, twenty of
 // the 98^3 MHD cavity 2135 -> 2086 us, a 40-step transient's gradient on 64^3
-// 4298 -> 4083 us.
+// 4298 -> 4110 us.
 template <class... P, class... A>
 cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t st, const A&... args)
 {

@@ -52,9 +52,11 @@ __device__ __forceinline__ F2 operator-(F2 a) { return F2(__fmul2_rn(a.v, make_f
 __device__ __forceinline__ F2& operator+=(F2& a, F2 b) { a = a + b; return a; }
 
 // One node in F2's arithmetic: both lanes hold it, so a node updated alone
-// gives the bits that it gives as half of a pair.  (Scalar __fadd_rn /
-// __fmul_rn in the same places do not: the packed operations' roundings are
-// not all theirs.)
+// gives the bits that it gives as half of a pair.  (Each packed operation
+// rounds as the scalar one does and no packed product and sum is contracted:
+// 2^20 random ones agree.  The whole update in __fadd_rn / __fmul_rn /
+// __fmaf_rn still gave other bits in F32 and F16 marches, so the difference is
+// one that the compiler makes across operations.)
 struct F1 {
     F2 w;
     __device__ __forceinline__ F1() {}
@@ -1320,7 +1322,7 @@ struct NodeIn {
     V ul0, ul1, ul2;   // low parts of the snapshot (b.snap_lo)
 };
 
-// FL_IN_F: the flow pass of a two-pass coupled update (coupled_induction_pass
+// FL_IN_F: the flow pass of a two-pass coupled update (induction_from_sources
 // wrote this step's Lorentz force into b.FL): the total force is the external
 // force plus b.FL, added as the one-pass update adds it.
 template <bool MHD, int MODE, bool FL_IN_F = false>
@@ -1559,8 +1561,9 @@ __device__ __forceinline__ void store_induction(const StepParams& p, const StepB
     b.FL[2 * N + n] = FLz;
 }
 
-// Pass 1 of the two-pass coupled update of node n from its inputs (loaded by the
-// caller, ahead of the gathers they are used after), rho, m and gathered g: the induction part, and the stores of g~ and of this step's Lorentz force.
+// Pass 1 of the two-pass coupled update of node n from its inputs (loaded by
+// the caller, ahead of the gathers they are used after), rho, m and gathered g:
+// the induction part, and the stores of g~ and of this step's Lorentz force.
 template <int ST, bool PACK>
 __device__ __forceinline__ void induction_from_sources(const StepParams& p, const StepBuffers& b, uint32_t n,
                                                       const NodeIn<float>& in, float rho_inv, float mx, float my,
@@ -1590,8 +1593,8 @@ __device__ __forceinline__ void node_from_sources(const StepParams& p, const Ste
     const size_t N = p.N;
     float om[19], og[21];
     NodeState<float> ns;
-    node_update<float, ST, MHD, COLL, PACK>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz, MODE != MODE_FIELDS, om,
-                                og, ns);
+    node_update<float, ST, MHD, COLL, PACK>(p, d, dl, q, ql, in.FLx, in.FLy, in.FLz, in.Fx, in.Fy, in.Fz,
+                                            MODE != MODE_FIELDS, om, og, ns);
 
     if (MODE == MODE_FIELDS) {
         if (fo.rho) fo.rho[n] = ns.rho;
@@ -2229,7 +2232,8 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
         if (p.cavity) {   // fluid box and / or moving lid: the one-node cavity kernel
             const unsigned grid = (unsigned)(((size_t)p.N + STEP_THREADS - 1) / STEP_THREADS);
             if (MODE != MODE_FIELDS && p.collision == 1) {
-                if constexpr (ST == ST_F32) e = launch_overlapped(cavity_kernel<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
+                if constexpr (ST == ST_F32)
+                    e = launch_overlapped(cavity_kernel<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
             } else if (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS && p.variant == 0) {
                 if constexpr (MHD && (ST == ST_F32 || ST == ST_F32C) && MODE != MODE_FIELDS) {
                     static const long long wave = resident_wave(cavity_kernel_coupled2<ST, MODE>, STEP_THREADS);
@@ -2246,7 +2250,8 @@ cudaError_t launch_mode(const StepParams& p, const StepBuffers& b_in, const Fiel
     if constexpr (MODE != MODE_FIELDS && (ST == ST_F32 || ST == ST_F32C || ST == ST_BF16)) {
         if (p.collision != 0) {   // preconditioned SRT-LBE: one node per thread
             const unsigned grid = (unsigned)(((size_t)p.N + STEP_THREADS - 1) / STEP_THREADS);
-            if (p.collision == 1) e = launch_overlapped(step_kernel_srt<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
+            if (p.collision == 1)
+                e = launch_overlapped(step_kernel_srt<ST, MHD, MODE, 1>, grid, STEP_THREADS, st, p, b, fo);
             else e = launch_overlapped(step_kernel_srt<ST, MHD, MODE, 2>, grid, STEP_THREADS, st, p, b, fo);
             if (nblocks) *nblocks = grid;
             return e;
