@@ -110,8 +110,10 @@ glbe_status glbe2d_set_force(glbe2d_ctx* ctx, const float* d_F);
 
 /* Advances n >= 0 steps; the step colliding a level t with t % 10 == 0 also
  * evaluates the residual.  With the automatic kernel form, small grids take
- * many steps in one launch, as in glbe_step_n: n >= 2 on up to 4096 nodes, and
- * with F32C storage and induction n >= 5 on 8192 to about 39,000. */
+ * many steps in one launch, as in glbe_step_n: n >= 2 on up to 4096 nodes, n >= 5
+ * on 8192 to about 77,000 with F32C storage or induction (F32 from 12,544), and
+ * n >= 40 on 32,768 to about 77,000 for the F32 and BF16 flow lattices, whose
+ * solves past 4096 nodes replay launches. */
 glbe_status glbe2d_step_n(glbe2d_ctx* ctx, long n);
 
 /* As glbe_set_barrier_test. */

@@ -947,25 +947,34 @@ constexpr int dense2d_blocks()
 // arithmetic bit for bit.
 // Table rows: the source node of each D2Q9 direction (the node itself where
 // the link is bounced) and the bounced-link bits; the D2Q5 directions share
-// the sources of the axis directions.  One cluster (up to 4096 nodes) wins in
-// every form; past it only the coupled F32C grids of 8192 nodes and more do,
-// against launches that overlap (us a step, launched -> resident; in brackets
-// the cooperative forms that are not built):
-//               F32 flow        F32 coupled     F32C coupled    BF16 coupled
-//   64 x 64     2.5 -> 1.75     3.1 -> 2.4      3.9 -> 2.9      3.2 -> 2.0
-//   80 x 80     2.5 -> (3.1)    3.1 -> (3.5)    4.0 -> (4.0)    3.2 -> (3.3)
-//   128 x 128   2.7 -> (3.0)    3.6 -> (3.45)   5.3 -> 3.9      3.8 -> (3.3)
-//   192 x 192   3.6 -> (3.1)    5.3 -> (3.6)    5.6 -> 4.0      4.2 -> (3.4)
-//   384 x 384   5.1 -> (5.6)    5.9 -> (7.2)    8.4 -> (11.7)   5.3 -> (6.4)
-// and solves of 200 steps, whose launches a graph replays (us):
-//   80 x 80     583 -> (684)    668 -> (780)    838 -> (875)    710 -> (744)
-//   128 x 128   585 -> (681)    713 -> (775)    950 -> 868      688 -> (751)
-//   192 x 192   620 -> (707)    787 -> (802)   1111 -> 879      827 -> (755)
-// (past 38,912 nodes, one tile on each SM, F32C coupled solves gained 1 to 4 %
-// up to 256 x 256 and lost 11 % at 288 x 288).
+// the sources of the axis directions.  One cluster (up to 4096 nodes) beats
+// launches that overlap in every form; past it the lines are RES2_LEAST and
+// resident2d_plan_t's.  A step of long marches (us, launched -> resident; in
+// brackets where the launches are taken) and a solve of 200 steps, whose
+// launches a graph replays:
+//               F32 flow        F32 coupled    F32C flow     F32C coupled   BF16 coupled
+//   64 x 64     2.5 -> 1.75     3.1 -> 2.4     3.0 -> 2.0    3.9 -> 2.9     3.2 -> 2.0
+//   80 x 80     2.5 -> (3.1)    3.1 -> (3.5)   3.1 -> (3.2)  4.0 -> (3.9)   3.3 -> (3.3)
+//   128 x 128   2.8 -> (3.1)    3.7 -> 3.4     3.6 -> 3.0    5.3 -> 3.9     3.9 -> 3.0
+//   192 x 192   3.7 -> 2.9      5.4 -> 3.4     4.7 -> 3.2    5.6 -> 3.9     4.2 -> 3.1
+//   256 x 256   4.2 -> 3.5      5.1 -> 4.1     5.3 -> 3.7    6.2 -> 5.1     4.5 -> 3.8
+//   288 x 288   4.9 -> (4.6)    5.8 -> (5.8)   5.3 -> (5.4)  6.7 -> (7.4)   5.4 -> (5.2)
+//   a solve on
+//   128 x 128   584 -> (679)    733 -> 742     705 -> 669    950 -> 848     754 -> 675
+//   192 x 192   620 -> (687)    798 -> 751     781 -> 711    1111 -> 860    831 -> 700
+//   256 x 256   789 -> (801)   1034 -> 911     958 -> 825    1276 -> 1106   950 -> 849
+//   288 x 288   951 -> (1006)  1197 -> (1252) 1122 -> (1159) 1393 -> (1569) 1110 -> (1119)
+// Held to two blocks an SM no form spills; held to 64 or 80 registers for several
+// tiles a block, 208 x 208 to 272 x 272 coupled F32 and F32C took 12 to 16 % longer.
 // ---------------------------------------------------------------------------
 constexpr int RES2_ROWS = 10;
-constexpr uint32_t RES2_LEAST = 8192;     // nodes of the cooperative form, at least
+// The cooperative form: nodes at least (below, launched steps are faster), and
+// two tiles on an SM at most (with a third the march is slower: 288 x 288).  The
+// plain flow forms' launches are so short that solves replay them whatever the
+// size and that only long marches of the larger of these grids gain (192 x 192
+// F32: 31 steps make up for the launch).
+constexpr uint32_t RES2_LEAST = 8192, RES2_LEAST_F32_MHD = 12544, RES2_LEAST_PLAIN_FLOW = 32768;
+constexpr long RES2_LEAST_STEPS_PLAIN_FLOW = 40;
 __host__ __device__ constexpr int axis9(int a5) { return a5 == 0 ? 0 : (a5 == 1 ? 1 : (a5 == 2 ? 3 : (a5 == 3 ? 2 : 4))); }
 static_assert(ex9(axis9(2)) == ex5(2) && ey9(axis9(3)) == ey5(3), "D2Q5 directions among the D2Q9 ones");
 
@@ -1037,7 +1046,7 @@ __device__ __forceinline__ void resident_update2(const P2& p, const B2& b, int n
 // the launched reduction's order, in the other a block's partials first, so
 // that a level's sums are one number per block.
 template <int ST, bool MHD, bool CLUSTER>
-__global__ void __launch_bounds__(RES_THREADS, 1) resident2d_kernel(const P2 p, const ResidentMarch m)
+__global__ void __launch_bounds__(RES_THREADS, CLUSTER ? 1 : 2) resident2d_kernel(const P2 p, const ResidentMarch m)
 {
     constexpr int GROUP = T2D / 32;
     extern __shared__ uint32_t slots[];          // [RES2_ROWS][blockDim.x]
@@ -1157,20 +1166,25 @@ cudaError_t resident2d_plan_t(uint32_t N, ResidentPlan* out)
 {
     constexpr size_t tile = (size_t)RES2_ROWS * RES_THREADS * sizeof(uint32_t);
     using K = void (*)(P2, ResidentMarch);
-    const K cluster = resident2d_kernel<ST, MHD, true>;
-    K coop = nullptr;
-    ResidentOcc oc{};
-    if constexpr (ST == GLBE_F32C && MHD) {
-        coop = resident2d_kernel<ST, MHD, false>;
-        static const ResidentOcc occ = resident_occupancy(coop, tile);
-        if (N >= RES2_LEAST) oc = occ;
-    }
+    const K cluster = resident2d_kernel<ST, MHD, true>, coop = resident2d_kernel<ST, MHD, false>;
+    constexpr bool PLAIN_FLOW = !MHD && ST != GLBE_F32C;
+    constexpr uint32_t LEAST = PLAIN_FLOW ? RES2_LEAST_PLAIN_FLOW : MHD && ST == GLBE_F32 ? RES2_LEAST_F32_MHD : RES2_LEAST;
+    static const ResidentOcc occ = [&] {
+        ResidentOcc o = resident_occupancy(coop, tile);
+        o.n[1] = o.n[1] < 2 ? o.n[1] : 2;
+        return o;
+    }();
     static const bool fits = [&] {
         cudaFuncSetAttribute(cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return resident_cluster_fits(cluster, tile);
     }();
-    return resident_plan_of(cluster, coop, K(nullptr), N, N, RES2_ROWS, RES_MAX_TILES * tile, oc, ResidentOcc{}, fits,
-                            out);
+    const cudaError_t e = resident_plan_of(cluster, coop, K(nullptr), N, N, RES2_ROWS, RES_MAX_TILES * tile,
+                                           N >= LEAST ? occ : ResidentOcc{}, ResidentOcc{}, fits, out);
+    if (PLAIN_FLOW && out->form == 2) {
+        out->least = RES2_LEAST_STEPS_PLAIN_FLOW;
+        out->solves = 0;
+    }
+    return e;
 }
 
 template <int ST>
@@ -1179,14 +1193,17 @@ cudaError_t resident2d_plan(bool mhd, uint32_t N, ResidentPlan* out)
     return mhd ? resident2d_plan_t<ST, true>(N, out) : resident2d_plan_t<ST, false>(N, out);
 }
 
+template <int ST, bool MHD>
+cudaError_t resident2d_march_t(const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
+{
+    return pl.form == 1 ? resident_launch(resident2d_kernel<ST, MHD, true>, pl, st, p, m)
+                        : resident_launch(resident2d_kernel<ST, MHD, false>, pl, st, p, m);
+}
+
 template <int ST>
 cudaError_t resident2d_march(bool mhd, const P2& p, const ResidentMarch& m, const ResidentPlan& pl, cudaStream_t st)
 {
-    if constexpr (ST == GLBE_F32C) {
-        if (pl.form == 2) return resident_launch(resident2d_kernel<ST, true, false>, pl, st, p, m);
-    }
-    return mhd ? resident_launch(resident2d_kernel<ST, true, true>, pl, st, p, m)
-               : resident_launch(resident2d_kernel<ST, false, true>, pl, st, p, m);
+    return mhd ? resident2d_march_t<ST, true>(p, m, pl, st) : resident2d_march_t<ST, false>(p, m, pl, st);
 }
 
 // Two x-adjacent nodes per thread (x periodic, even nx; FP32 or BF16
@@ -2113,7 +2130,7 @@ glbe_status glbe2d_solve(glbe2d_ctx* c, double tol, long max_steps, long* steps_
         if (t % 10 == 0) snap = t;
     glbe_status s = lead > 0 ? glbe2d_step_n(c, lead) : GLBE_OK;
     if (s != GLBE_OK) return s;
-    const bool resident = c->res.form != 0;
+    const bool resident = c->res.form && c->res.solves;
     if (!resident) s = build_chunk2(c);
     if (s != GLBE_OK) return s;
     ctl2d_kernel<<<1, 1, 0, c->stream>>>(nullptr, 0, c->stop_dev, 0, c->tol_dev, tol, nullptr, nullptr, 0);

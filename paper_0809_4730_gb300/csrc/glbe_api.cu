@@ -902,7 +902,7 @@ glbe_status glbe_solve(glbe_ctx* c, double tol, long max_steps, long* steps_out,
         if (s != GLBE_OK) return s;
     }
     glbe_status s = GLBE_OK;
-    const bool resident = c->res.form != 0;
+    const bool resident = c->res.form && c->res.solves;
     if (!resident) s = build_chunk(c);
     if (s != GLBE_OK) return s;
     misc_set_kernel<<<1, 1, 0, c->stream>>>(nullptr, 0, c->stop_dev, 0, c->tol_dev, tol, nullptr, nullptr, 0);

@@ -218,13 +218,16 @@ struct ResidentPlan {
     int pair;             // two nodes per thread
     int blocks, threads;
     unsigned smem;
+    long least;           // steps of glbe_step_n that are marched so, at least
+    int solves;           // solves march so, too (else they replay launches)
 };
-// Whether n steps are marched so.  A cooperative launch, its tables and the look
-// at its flag when the host next waits cost as much as some four launched steps
-// save: two F32 steps of 64^3 and a wait took 57 us so and 45 launched, four 75
-// and 63, eight 111 and 105 (40^3: 47 and 36, 55 and 46, 72 and 72); a cluster's
-// two steps cost what two launched ones do (4 x 32 x 4: 37 and 36 us).
-inline bool resident_takes(const ResidentPlan& pl, long n) { return pl.form == 1 ? n >= 2 : pl.form && n >= 5; }
+// The shortest marches.  A cooperative launch, its tables and the look at its flag
+// when the host next waits cost as much as some four launched steps save: two
+// F32 steps of 64^3 and a wait took 57 us so and 45 launched, four 75 and 63,
+// eight 111 and 105 (40^3: 47 and 36, 55 and 46, 72 and 72); a cluster's two steps
+// cost what two launched ones do (4 x 32 x 4: 37 and 36 us).
+constexpr long RES_LEAST_CLUSTER = 2, RES_LEAST_COOP = 5;
+inline bool resident_takes(const ResidentPlan& pl, long n) { return pl.form && n >= pl.least; }
 template <int ST>
 cudaError_t resident_plan(bool mhd, const StepParams& p, ResidentPlan* out);
 template <int ST>

@@ -140,7 +140,7 @@ bool resident_cluster_fits(K kernel, size_t tile_bytes)
 inline ResidentPlan resident_cluster_plan(uint32_t N, int rows)
 {
     const int threads = 32 * (int)((N + RES_CLUSTER * 32 - 1) / (RES_CLUSTER * 32));
-    return {1, 0, RES_CLUSTER, threads, (unsigned)(rows * threads * sizeof(uint32_t))};
+    return {1, 0, RES_CLUSTER, threads, (unsigned)(rows * threads * sizeof(uint32_t)), RES_LEAST_CLUSTER, 1};
 }
 
 // A cooperative form for `units` updates: the fewest tiles per block (at most
@@ -155,7 +155,7 @@ inline bool resident_grid_plan(const ResidentOcc& occ, uint32_t units, int sms, 
     for (int per = 1; per <= max_per && occ.n[per] == occ.n[1] && occ.n[1] * per * tile_bytes <= table_bytes; ++per) {
         const long long room = (long long)occ.n[1] * sms;
         if (room * per < tiles) continue;
-        *out = {form, 0, (int)(room < tiles ? room : tiles), RES_THREADS, (unsigned)(per * tile_bytes)};
+        *out = {form, 0, (int)(room < tiles ? room : tiles), RES_THREADS, (unsigned)(per * tile_bytes), RES_LEAST_COOP, 1};
         return true;
     }
     return false;

@@ -17,9 +17,14 @@ SIZES = [((86, 86, 84), "yz", "f32", False, True), ((88, 86, 84), "yz", "f32", F
          ((68, 67, 68), "y", "f32", True, True), ((68, 68, 68), "y", "f32", True, False),          # coupled
          ((68, 67, 68), "y", "f32c", True, True), ((68, 68, 68), "y", "f32c", True, False),
          ((62, 61, 61), "y", "bf16", True, True), ((62, 62, 62), "y", "bf16", True, False)]
-SIZES2 = [((90, 91), dict(), False), ((91, 91), dict(), True), ((197, 197), dict(), True), ((198, 197), dict(), False),
-          ((128, 128), dict(storage="f32"), False), ((128, 128), dict(storage="bf16"), False),
-          ((128, 128), dict(induction=0), False), ((700, 700), dict(storage="bf16", induction=0), False)]
+SIZES2 = [((90, 91), dict(), False), ((91, 91), dict(), True), ((278, 279), dict(), True), ((279, 279), dict(), False),
+          ((91, 91), dict(induction=0), True), ((279, 279), dict(induction=0), False),
+          ((91, 91), dict(storage="bf16"), True), ((279, 279), dict(storage="bf16"), False),
+          ((112, 111), dict(storage="f32"), False), ((112, 112), dict(storage="f32"), True),
+          ((278, 279), dict(storage="f32"), True), ((279, 279), dict(storage="f32"), False),
+          ((181, 181), dict(storage="bf16", induction=0), False), ((182, 181), dict(storage="bf16", induction=0), True),
+          ((278, 279), dict(storage="f32", induction=0), True), ((279, 279), dict(storage="f32", induction=0), False),
+          ((700, 700), dict(storage="bf16", induction=0), False)]
 
 
 def _meets(S):
@@ -35,9 +40,9 @@ def _meets(S):
 def _compare(A, B, start):
     start(A)
     start(B)
-    for n in (4, 5, 13):
+    for n in (4, 5, 13, 39, 40):
         A.step(n)
-    for _ in range(22):
+    for _ in range(101):
         B.step(1)
     A.sync()
     _same(A.get_state(), B.get_state())
@@ -63,16 +68,20 @@ def test_2d_lines(shape, kw, meets):
     _compare(A, B, _state2)
 
 
-@pytest.mark.parametrize("two_d", [False, True])
-def test_four_steps_are_launched_and_five_march(two_d):
+@pytest.mark.parametrize("make,start,least", [(lambda: _solver((48, 48, 48), "y", "f32", False), _start, 5),
+                                             (lambda: _solver2(), _state2, 5),
+                                             (lambda: _solver2((200, 200), storage="f32", induction=0), _state2, 40)])
+def test_the_shortest_march(make, start, least):
     """Where the blocks meet at the counting barrier: with one of them absent, only a march runs out."""
     from paper_0809_4730_gb300.glbe import GLBE_ERR_TIMEOUT
-    S = _solver2() if two_d else _solver((48, 48, 48), "y", "f32", False)
-    (_state2 if two_d else _start)(S)
+    S = make()
+    start(S)
     S.set_barrier_test(LIMIT, 0)
-    for n in (0, 1, 2, 3, 4):
+    for n in (0, 1, 2, 3, least - 1):
         S.step(n)
         S.sync()
-    S.step(5)
+    if least == 40:
+        assert S.solve(1e-30, 100)[0] == GLBE_ERR_TIMEOUT      # its step limit: a solve of these replays launches
+    S.step(least)
     assert _status(S.sync) == GLBE_ERR_TIMEOUT
     S.close()
